@@ -57,8 +57,10 @@ typedef enum {
     VPLBM_EIO = 8            /* file read or write failed */
 } vplbm_status;
 
-/* Storage precision of the populations.  Arithmetic is FP64 for VPLBM_F64
- * and FP32 otherwise.  The force/torque sums are FP64 for VPLBM_F64 and
+/* Storage precision of the populations.  Arithmetic is 64-bit for VPLBM_F64
+ * (the MRT update of a node near rho0 in 64-bit fixed point, whose error is
+ * below that of the FP64 instructions; FP64 instructions for any other node
+ * and for BGK) and FP32 otherwise.  The force/torque sums are FP64 for VPLBM_F64 and
  * float-float (about 44 bits, converted exactly to FP64) otherwise; the body
  * update is always FP64.  The _DEV variants store f_a - w_a rho0 (deviation
  * from rest). */
@@ -272,8 +274,10 @@ vplbm_status vplbm_get_body_k(vplbm_ctx *ctx, int k, double q[3], double v[3], l
  *                          into registers (every precision), register budget
  *                          of 4 blocks of 256 threads per SM (64 registers):
  *                          the default for FP64 storage;
- *  VPLBM_KERNEL_SCALAR_48  the same sized for 5 blocks (48 registers);
- *  VPLBM_KERNEL_SCALAR_40  the same sized for 6 blocks (40 registers): the
+ *  VPLBM_KERNEL_SCALAR_48  the same sized for 5 blocks (48 registers; FP64
+ *                          storage: 3 blocks, 80 registers);
+ *  VPLBM_KERNEL_SCALAR_40  the same sized for 6 blocks (40 registers; FP64
+ *                          storage: 2 blocks, 128 registers): the
  *                          default for FP32 / FP16 storage (256 x 1 blocks);
  *  VPLBM_KERNEL_TMA        persistent blocks fed by tensor-memory-accelerator
  *                          copies into a shared-memory ring (FP32/FP16

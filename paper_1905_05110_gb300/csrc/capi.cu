@@ -484,6 +484,7 @@ vplbm_status setup(vplbm_ctx *c, const vplbm_lattice_desc *lat, const vplbm_body
     p.pen_kf = (float)p.pen_k;
     fold_consts(p.pc, lat->s, lat->gx, lat->gy);
     fold_consts(p.pcd, lat->s, lat->gx, lat->gy);
+    fold_fixed(p.fx, lat->s, lat->rho0, lat->gx, lat->gy, p.pen_k);
     // wall velocity profiles: [side][comp][maxlen]
     const int maxlen = lat->nx > lat->ny ? lat->nx : lat->ny;
     const size_t nprof = (size_t)8 * maxlen;

@@ -1,0 +1,344 @@
+// The FP64 path's MRT update in 64-bit fixed point on the integer pipes.
+//
+// What bounds it: GB300 issues two FP64 lanes per clock and SM, so the 111
+// FP64 instructions of the update kept that pipe busy for 55 clocks per node
+// and nothing else mattered (4.1 k MLUPS on 2048 x 1024, 9 % of the HBM
+// rate).  The integer pipes are 32 to 64 times as wide, and a node's
+// populations share one scale (they are fractions of rho ~ rho0), so the
+// update runs on integers: additions are exact, a product is three 32-bit
+// wide multiplies, and the collision is written as f + M^-1 (dm), which
+// needs six products with the relaxation rates, five for the velocity and
+// the quadratic terms, and one reciprocal.
+//
+// Numbers.  A population f is the integer x = f 2^(59 - E), 2^E >= rho0 >
+// 2^(E-1): the grid is 2^-59 of that scale, at or below the spacing of the
+// doubles it is read from for f >= 2^(E-7) (an ordinary diagonal population
+// is rho0 / 36), so the read is exact there.  Every product is rounded to
+// the nearest grid point (plus at most one more unit), the results are
+// rounded to doubles to nearest even.  The collision's increments conserve
+// mass, and without forcing momentum, exactly.  Its error against exact
+// arithmetic is a third of that of the FP64 instructions it replaces (RMS
+// over the populations of an update at rho0 = 1, in 113-bit arithmetic:
+// 0.7e-17 against 2.2e-17, most of it the final rounding to double).
+//
+// Measured (GB300, us per step, best block shape): 2048 x 1024 513 -> 63.5
+// (32.9 k MLUPS, 4.7 TB/s), 256 x 128 28 -> 13.5 (there the launch boundary
+// and the body's sums remain).
+//
+// Range.  A node takes this path if every population is in
+// [2^(E-32), 2^E), rho in [2^(E-1), 1.5 2^E), |j| < 0.35 2^E and (body
+// nodes) the slip |u_s - v| < 1/4, and if every result is at least
+// 2^(E-27); sums and products then stay below 2^63.  Any other node (a
+// negative population, a density far from rho0, NaN, infinities) takes the
+// FP64 instructions, which accept everything.
+#pragma once
+
+#include <math.h>
+#include <stdint.h>
+#include <string.h>
+
+#if defined(__CUDACC__)
+#define VPLBM_FX __host__ __device__ __forceinline__
+#else
+#define VPLBM_FX inline
+#endif
+
+namespace vplbm {
+namespace {
+
+// A factor r in (-1/2, 1/2) as r = hi 2^-32 + lo 2^-64 with signed digits.
+struct FxFactor {
+    int hi, lo;
+};
+
+// Host-folded constants of the fixed-point update (uniform over a run).
+struct FixedConsts {
+    int ok;                     // the run's rho0 and g are in range
+    int e;                      // E
+    double unit;                // 2^(E - 59)
+    unsigned hi_min, hi_max;    // high words of the doubles in [2^(E-32), 2^E)
+    FxFactor r1, r2, r4, r6, r7, r8;   // s1/36, s2/12, s4/12, s6/12, s7/4, s8/4
+    // forcing: (1 - s/2) / 6 for e and eps, / 12 for q, / 2 and / 4 for the
+    // stress, 1/6, and pen_k / 4
+    FxFactor h1, h2, h4, h6, h7, h8, sixth, k4;
+    long long gvx, gvy;         // g 2^60
+    int forced;                 // g is not zero
+};
+
+inline FxFactor fx_factor(double r)
+{
+    const long long v = llrint(ldexp(r, 64));
+    FxFactor f;
+    f.lo = (int)(uint32_t)(uint64_t)v;
+    f.hi = (int)((v - (long long)f.lo) >> 32);
+    return f;
+}
+
+inline void fold_fixed(FixedConsts &k, const double *s, double rho0, double gx, double gy, double pen_k)
+{
+    memset(&k, 0, sizeof k);
+    int e = 0;
+    const double m = frexp(rho0, &e);   // rho0 = m 2^e, m in [1/2, 1)
+    if (m == 0.5) e -= 1;               // rho0 in (2^(E-1), 2^E]
+    if (!(rho0 > 0.0) || e < -400 || e > 400 || !(fabs(gx) < 0.0625) || !(fabs(gy) < 0.0625)) return;
+    k.ok = 1;
+    k.e = e;
+    k.unit = ldexp(1.0, e - 59);
+    k.hi_min = (unsigned)(991 + e) << 20;
+    k.hi_max = (unsigned)(1023 + e) << 20;
+    k.r1 = fx_factor(s[1] / 36.0); k.r2 = fx_factor(s[2] / 12.0); k.r4 = fx_factor(s[4] / 12.0);
+    k.r6 = fx_factor(s[6] / 12.0); k.r7 = fx_factor(s[7] / 4.0); k.r8 = fx_factor(s[8] / 4.0);
+    k.h1 = fx_factor((1.0 - 0.5 * s[1]) / 6.0); k.h2 = fx_factor((1.0 - 0.5 * s[2]) / 6.0);
+    k.h4 = fx_factor((1.0 - 0.5 * s[4]) / 12.0); k.h6 = fx_factor((1.0 - 0.5 * s[6]) / 12.0);
+    k.h7 = fx_factor((1.0 - 0.5 * s[7]) / 2.0); k.h8 = fx_factor((1.0 - 0.5 * s[8]) / 4.0);
+    k.sixth = fx_factor(1.0 / 6.0);
+    k.k4 = fx_factor(0.25 * pen_k);     // pen_k = 1 / (eta + 1/2) < 2
+    k.gvx = llrint(ldexp(gx, 60));
+    k.gvy = llrint(ldexp(gy, 60));
+    k.forced = gx != 0.0 || gy != 0.0;
+}
+
+VPLBM_FX int fx_clz(uint32_t x)
+{
+#if defined(__CUDA_ARCH__)
+    return __clz((int)x);
+#else
+    return x ? __builtin_clz(x) : 32;
+#endif
+}
+
+VPLBM_FX uint64_t fx_bits(double d)
+{
+#if defined(__CUDA_ARCH__)
+    return (uint64_t)__double_as_longlong(d);
+#else
+    uint64_t b;
+    memcpy(&b, &d, 8);
+    return b;
+#endif
+}
+
+VPLBM_FX double fx_double(uint64_t b)
+{
+#if defined(__CUDA_ARCH__)
+    return __longlong_as_double((long long)b);
+#else
+    double d;
+    memcpy(&d, &b, 8);
+    return d;
+#endif
+}
+
+VPLBM_FX FxFactor fx_split(long long r)
+{
+    FxFactor f;
+    f.lo = (int)(uint32_t)(uint64_t)r;
+    f.hi = (int)(r >> 32) + (int)((uint32_t)f.lo >> 31);
+    return f;
+}
+
+// x r to the nearest integer but for the product of the two low digits
+// (below half a unit); |x| < 2^63.
+VPLBM_FX long long fx_mul(long long x, FxFactor r)
+{
+    const FxFactor a = fx_split(x);
+    const long long m = (long long)a.lo * r.hi + 0x80000000LL + (long long)a.hi * r.lo;
+    return (long long)a.hi * r.hi + (m >> 32);
+}
+
+// The double with bits b, in [2^(E-32), 2^E), on the grid (truncated).
+VPLBM_FX long long fx_from(uint64_t b, int e)
+{
+    const uint32_t hi = (uint32_t)(b >> 32), lo = (uint32_t)b;
+    const uint32_t s = (uint32_t)(1022 + e) - (hi >> 20);   // 0 .. 31 in range
+    const uint32_t mh = (((hi << 6) | (lo >> 26)) & 0x3ffffffu) | 0x4000000u, ml = lo << 6;
+#if defined(__CUDA_ARCH__)
+    const uint32_t rl = __funnelshift_r(ml, mh, s), rh = mh >> (s & 31);
+#else
+    const uint64_t m = ((((uint64_t)mh) << 32) | ml) >> (s & 31);
+    const uint32_t rl = (uint32_t)m, rh = (uint32_t)(m >> 32);
+#endif
+    return (long long)(((uint64_t)rh << 32) | rl);
+}
+
+// The grid point x in [2^32, 2^61) as a double, to nearest even.
+VPLBM_FX double fx_to(long long x, int e)
+{
+    const uint32_t hi = (uint32_t)((uint64_t)x >> 32), lo = (uint32_t)(uint64_t)x;
+    const uint32_t n = (uint32_t)fx_clz(hi) - 1;   // leading bit to bit 62
+#if defined(__CUDA_ARCH__)
+    const uint32_t yh = __funnelshift_l(lo, hi, n), yl = lo << (n & 31);
+#else
+    const uint64_t yy = ((((uint64_t)hi) << 32) | lo) << n;
+    const uint32_t yh = (uint32_t)(yy >> 32), yl = (uint32_t)yy;
+#endif
+    uint64_t y = ((uint64_t)yh << 32) | yl;
+    y += 0x1ffu + ((yl >> 10) & 1u);
+    y >>= 10;
+    return fx_double(y + ((uint64_t)((uint32_t)(1025 + e - (int)n) << 20) << 32));
+}
+
+// 2^120 / rho for rho in [2^58, 2^60), relative error below 2^-60: a 32-bit
+// estimate from the FP32 reciprocal, then 1 / (1 - d) = 1 + d + d^2 with the
+// exact residual d.
+VPLBM_FX long long fx_recip(long long rho)
+{
+    const uint32_t rh = (uint32_t)((uint64_t)rho >> 32), rl = (uint32_t)(uint64_t)rho;
+    const float rf = (float)(uint32_t)((uint64_t)rho >> 28);   // rho 2^-28
+#if defined(__CUDA_ARCH__)
+    float inv;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv) : "f"(rf));
+#else
+    const float inv = 1.0f / rf;
+#endif
+    const uint32_t r0 = (uint32_t)(inv * 1152921504606846976.0f);   // 2^60 / (rho 2^-28) = 2^88 / rho
+    // 2^88 - rho r0 in units of 2^16: |d| 2^72 < 2^52
+    const uint64_t pl = (uint64_t)rl * r0;
+    const uint64_t ph = (uint64_t)rh * r0 + (pl >> 32);
+    long long d = -(long long)((ph << 16) | ((uint32_t)pl >> 16));
+    const long long dh = (int)(d >> 32);
+    d += (dh * dh) >> 8;
+    const long long lo = (long long)((uint64_t)r0 * (uint32_t)(uint64_t)d >> 32);
+    return (long long)((uint64_t)r0 << 32) + (((long long)(int)(d >> 32) * (long long)r0 + lo) >> 8);
+}
+
+// The part of the update that a penalized node (or a lattice under a uniform
+// acceleration) does differently, a function of its own on the device: few
+// nodes take it, and inlined it costs the others registers.  In: the moments
+// (v: velocity times 2^61) and the solid velocity us; out: the increments
+// along the rows of M and G / 6, and a 2^60 of the penalization.  False if
+// the slip is out of range.
+struct FxForced {
+    long long rho, jx, jy, vx, vy, usx, usy, f0, sa, sd, qx, qy, pxx, pxy;   // in
+    long long de, dep, dqx, dqy, dp, dr, gx6, gy6, ax, ay;                   // out
+};
+
+#if defined(__CUDACC__)
+__device__ __noinline__
+#else
+inline
+#endif
+bool fx_forced(const FixedConsts &k, bool chi, FxForced &w)
+{
+    const long long wx = w.vx + k.gvx, wy = w.vy + k.gvy;   // v = j / rho + g / 2
+    long long ax = 0, ay = 0;                               // a 2^60
+    if (chi) {
+        const long long lx = w.usx - wx, ly = w.usy - wy;
+        constexpr long long Q = 1LL << 59;
+        if ((uint64_t)(lx + Q) >= (uint64_t)(2 * Q) || (uint64_t)(ly + Q) >= (uint64_t)(2 * Q)) return false;
+        ax = fx_mul(2 * lx, k.k4);
+        ay = fx_mul(2 * ly, k.k4);
+    }
+    const FxFactor ux = fx_split(wx + ax), uy = fx_split(wy + ay);   // u = v + a / 2
+    const long long r8 = (long long)((uint64_t)w.rho << 3);
+    const long long Gx = fx_mul(r8, fx_split(2 * (ax + k.gvx))), Gy = fx_mul(r8, fx_split(2 * (ay + k.gvy)));
+    const long long mx = w.jx + (Gx >> 1), my = w.jy + (Gy >> 1);    // rho u = j + G / 2
+    const long long mx8 = (long long)((uint64_t)mx << 3), my8 = (long long)((uint64_t)my << 3);
+    const long long A = fx_mul(mx8, ux), B = fx_mul(my8, uy), C = fx_mul(mx8, uy);
+    const long long Gx8 = (long long)((uint64_t)Gx << 3), Gy8 = (long long)((uint64_t)Gy << 3);
+    const long long xx = fx_mul(Gx8, ux), yy = fx_mul(Gy8, uy), xy = fx_mul(Gy8, ux) + fx_mul(Gx8, uy);
+    const long long K = A + B;
+    w.de = fx_mul(2 * w.f0 - w.sa - 4 * w.sd + 3 * K, k.r1) + fx_mul(xx + yy, k.h1);
+    w.dep = fx_mul(w.sa - w.f0 - K, k.r2) - fx_mul(xx + yy, k.h2);
+    w.dqx = fx_mul(w.qx - (Gx >> 1), k.r4) - fx_mul(Gx, k.h4);
+    w.dqy = fx_mul(w.qy - (Gy >> 1), k.r6) - fx_mul(Gy, k.h6);
+    w.dp = fx_mul(A - B - w.pxx, k.r7) + fx_mul(xx - yy, k.h7);
+    w.dr = fx_mul(C - w.pxy, k.r8) + fx_mul(xy, k.h8);
+    w.gx6 = fx_mul(Gx, k.sixth);
+    w.gy6 = fx_mul(Gy, k.sixth);
+    w.ax = ax;
+    w.ay = ay;
+    return true;
+}
+
+// One node: pulled populations f (bits of doubles) -> post-collision
+// populations out.  chi: the node is in a body of solid velocity us (times
+// 2^61).  Returns false (out untouched) if the node is out of range; rho and
+// a 2^60 (the penalization's acceleration) are kept for the body's sums.
+#if defined(__CUDACC__)
+__device__ __forceinline__
+#else
+inline
+#endif
+bool fx_update(const FixedConsts &k, const uint64_t fb[9], bool chi, long long usx, long long usy,
+                        double out[9], long long &rho_o, long long &ax_o, long long &ay_o)
+{
+    uint32_t top = 0, low = 0xffffffffu;
+    long long f[9];
+#if defined(__CUDA_ARCH__)
+#pragma unroll
+#endif
+    for (int a = 0; a < 9; ++a) {
+        const uint32_t hi = (uint32_t)(fb[a] >> 32);
+        top = hi > top ? hi : top;
+        low = hi < low ? hi : low;
+        f[a] = fx_from(fb[a], k.e);
+    }
+    bool ok = top < k.hi_max && low >= k.hi_min;
+    const long long d13 = f[1] - f[3], d24 = f[2] - f[4], b13 = f[1] + f[3], b24 = f[2] + f[4];
+    const long long d56 = f[5] - f[6], d87 = f[8] - f[7], a56 = f[5] + f[6], a78 = f[7] + f[8];
+    const long long sx = d56 + d87, ty = a56 - a78, sa = b13 + b24, sd = a56 + a78;
+    const long long rho = f[0] + sa + sd;
+    const long long jx = d13 + sx, jy = d24 + ty;
+    constexpr long long J = 201769274521386496LL;   // 0.35 2^59
+    ok = ok && (uint64_t)(rho - (1LL << 58)) < (uint64_t)(1LL << 59) && (uint64_t)(jx + J) < (uint64_t)(2 * J) &&
+         (uint64_t)(jy + J) < (uint64_t)(2 * J);
+    if (!ok) return false;
+    const FxFactor inv = fx_split(fx_recip(rho));
+    const long long vx = fx_mul((long long)((uint64_t)jx << 5), inv), vy = fx_mul((long long)((uint64_t)jy << 5), inv);   // u 2^61
+    long long de, dep, dqx = d13 - 2 * sx, dqy = d24 - 2 * ty, dp, dr;
+    long long gx6 = 0, gy6 = 0;
+    if (chi || k.forced) {
+        FxForced w;
+        w.rho = rho; w.jx = jx; w.jy = jy; w.vx = vx; w.vy = vy; w.usx = usx; w.usy = usy;
+        w.f0 = f[0]; w.sa = sa; w.sd = sd; w.qx = dqx; w.qy = dqy; w.pxx = b13 - b24; w.pxy = d56 - d87;
+        if (!fx_forced(k, chi, w)) return false;
+        de = w.de; dep = w.dep; dqx = w.dqx; dqy = w.dqy; dp = w.dp; dr = w.dr;
+        gx6 = w.gx6; gy6 = w.gy6;
+        ax_o = w.ax;
+        ay_o = w.ay;
+    } else {
+        const FxFactor ux = fx_split(vx), uy = fx_split(vy);
+        const long long jx8 = (long long)((uint64_t)jx << 3), jy8 = (long long)((uint64_t)jy << 3);
+        const long long A = fx_mul(jx8, ux), B = fx_mul(jy8, uy), C = fx_mul(jx8, uy);   // rho ux^2, uy^2, ux uy
+        const long long K = A + B;
+        de = fx_mul(2 * f[0] - sa - 4 * sd + 3 * K, k.r1);
+        dep = fx_mul(sa - f[0] - K, k.r2);
+        dqx = fx_mul(dqx, k.r4);
+        dqy = fx_mul(dqy, k.r6);
+        dp = fx_mul(A - B - (b13 - b24), k.r7);
+        dr = fx_mul(C - (d56 - d87), k.r8);
+    }
+    // M^-1 dm: the rows of Eq. (15) over their squared norms
+    const long long ax1 = -de - 2 * dep, dg = 2 * de + dep;
+    const long long x1 = gx6 - 2 * dqx, y1 = gy6 - 2 * dqy, x2 = gx6 + dqx, y2 = gy6 + dqy;
+    const long long p1 = ax1 + dp, p2 = ax1 - dp, q1 = dg + dr, q2 = dg - dr;
+    const long long s2 = x2 + y2, m2 = x2 - y2;
+    f[0] += 4 * (dep - de);
+    f[1] += p1 + x1;
+    f[3] += p1 - x1;
+    f[2] += p2 + y1;
+    f[4] += p2 - y1;
+    f[5] += q1 + s2;
+    f[7] += q1 - s2;
+    f[8] += q2 + m2;
+    f[6] += q2 - m2;
+    int lo = (int)(f[0] >> 32);
+#if defined(__CUDA_ARCH__)
+#pragma unroll
+#endif
+    for (int a = 1; a < 9; ++a) {
+        const int h = (int)(f[a] >> 32);
+        lo = h < lo ? h : lo;
+    }
+    if (lo < 1) return false;
+#if defined(__CUDA_ARCH__)
+#pragma unroll
+#endif
+    for (int a = 0; a < 9; ++a) out[a] = fx_to(f[a], k.e);
+    rho_o = rho;
+    return true;
+}
+
+}  // namespace
+}  // namespace vplbm

@@ -35,7 +35,7 @@ namespace {
 // writes, so they run before the wait on the previous step's grid
 // (programmatic dependent launch).
 template <int P, int COLL>
-__global__ void __launch_bounds__(256, 5) vp_mrt_step_batch(const BatchLaunch bl)
+__global__ void __launch_bounds__(256, P == VPLBM_F64 ? 4 : 5) vp_mrt_step_batch(const BatchLaunch bl)
 {
     __shared__ double red[8][NPART];
     __shared__ float rows[NPART - 1][256];

@@ -85,7 +85,7 @@ __device__ __forceinline__ void multi_tile(const StepParams &p, int tile_x, int 
 // blocks are [body_blocks[k], body_blocks[k + 1]); the first of them also
 // computes the next pose of body k when it moves on a prescribed path.
 template <int P, int MINB, int COLL>
-__global__ void __launch_bounds__(256, MINB) vp_mrt_step_multi(const StepParams p)
+__global__ void __launch_bounds__(256, budget_blocks<P>(MINB)) vp_mrt_step_multi(const StepParams p)
 {
     __shared__ double red[8][NPART];
     __shared__ float rows[NPART - 1][256];

@@ -51,7 +51,7 @@ __device__ __forceinline__ void scalar_tile(const StepParams &p, int tile_x, int
 }
 
 // MINB: blocks of 256 threads per SM the register budget is sized for
-// (4: 64 registers, 5: 48, 6: 40).
+// (4: 64 registers, 5: 48, 6: 40; FP64 storage: see budget_blocks).
 //
 // Launched with programmatic dependent launch: every block lets the next
 // step's grid start launching at once, and waits (in hardware) until the
@@ -68,7 +68,7 @@ __device__ __forceinline__ void scalar_tile(const StepParams &p, int tile_x, int
 // loads.  Body block 0 also computes the next pose of a body on a
 // prescribed path.
 template <int P, int MINB, int COLL, int SHAPE>
-__global__ void __launch_bounds__(256, MINB) vp_mrt_step(const StepParams p)
+__global__ void __launch_bounds__(256, budget_blocks<P>(MINB)) vp_mrt_step(const StepParams p)
 {
     __shared__ double red[8][NPART];
     __shared__ float rows[NPART - 1][256];

@@ -8,6 +8,7 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include "fixed64.cuh"
 #include "vplbm.h"
 
 namespace vplbm {
@@ -102,6 +103,7 @@ struct StepParams {
     float rho0f, gxf, gyf, pen_kf, r2f;
     FoldedConsts<float> pc;       // FP32 folded factors
     FoldedConsts<double> pcd;     // FP64 folded factors
+    FixedConsts fx;               // the FP64 kernel's fixed-point constants
     int bc[4];
     double wall_u0[4][2];
     const double *wall_prof[4][2];

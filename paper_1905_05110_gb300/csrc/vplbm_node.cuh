@@ -18,6 +18,14 @@ template <> struct Prec<VPLBM_F64> { using S = double; using T = double; static 
 template <> struct Prec<VPLBM_F32_DEV> { using S = float; using T = float; static constexpr bool DEV = true; };
 template <> struct Prec<VPLBM_F16_DEV> { using S = __half; using T = float; static constexpr bool DEV = true; };
 
+// Blocks of 256 threads per SM that a scalar step kernel's register budget is
+// sized for, from the budget asked for (4, 5 or 6).  The FP64 kernel's
+// fixed-point update holds nine 64-bit values and their sums: at 48 and 40
+// registers it would spill in the middle of the update, so those two choices
+// give it more registers instead (80 and 128).  us per step at 64, 80 and
+// 128 registers: 2048 x 1024 63.5, 64.1, 73.4; 256 x 128 14.2, 13.5, 13.1.
+template <int P> constexpr int budget_blocks(int minb) { return P != VPLBM_F64 || minb == 4 ? minb : minb == 5 ? 3 : 2; }
+
 // Loads of the populations and the pose written by the previous time step.
 // A kernel launched once per step reads them through the read-only path
 // (ld.global.nc: they do not change while it runs).  A kernel that runs
@@ -467,9 +475,9 @@ __device__ __forceinline__ void solid_node_terms(const StepParams &p, const type
 constexpr int SHAPE_ANY = -1;
 
 // chi of node (i, j) for one body (Eq. 2, Alg. 1 step 4) and its lever arm
-// (dxl, dyl) = x - x_G.  The storage kernels test in FP32 and re-test in
-// FP64 where the FP32 value is within the band of the boundary, so the
-// result is the exact FP64 predicate.  SHAPE: VPLBM_SHAPE_DISK, _ELLIPSE or
+// (dxl, dyl) = x - x_G (FP64 storage: of the solid nodes only).  Tested in
+// FP32 and re-tested in FP64 where the FP32 value is within the band of the
+// boundary, so the result is the exact FP64 predicate.  SHAPE: VPLBM_SHAPE_DISK, _ELLIPSE or
 // _RECTANGLE fixed at compile time, or SHAPE_ANY to read it from the body.
 template <int P, int SHAPE>
 __device__ __forceinline__ bool body_chi(const DevBody &body, float r2f, const BodyState *__restrict__ bs, int i,
@@ -478,7 +486,7 @@ __device__ __forceinline__ bool body_chi(const DevBody &body, float r2f, const B
     using T = typename Prec<P>::T;
     constexpr bool DEV = Prec<P>::DEV;
     bool chi = false;
-    if constexpr (DEV) {
+    {
         const int2 xy = VPLBM_LDG(reinterpret_cast<const int2 *>(&bs->xi));
         const float2 fr = VPLBM_LDG(reinterpret_cast<const float2 *>(&bs->xf));
         const float dxf = (float)(i - xy.x) - fr.x;
@@ -511,15 +519,16 @@ __device__ __forceinline__ bool body_chi(const DevBody &body, float r2f, const B
             if (fabsf(d2 - r2) <= band) chi = chi_exact(i, j, bs->q[0], bs->q[1], body.r2);
             else chi = d2 <= r2;
         }
-        dxl = dxf; dyl = dyf;
-    } else {
-        const double xg = VPLBM_LDG(&bs->q[0]), yg = VPLBM_LDG(&bs->q[1]);
-        const int shape = SHAPE == SHAPE_ANY ? body.shape : SHAPE;
-        chi = shape == VPLBM_SHAPE_ELLIPSE   ? chi_exact_ellipse(i, j, bs, body)
-              : shape == VPLBM_SHAPE_RECTANGLE ? chi_exact_rect(i, j, bs, body)
-                                               : chi_exact(i, j, xg, yg, body.r2);
-        dxl = (double)i - xg;
-        dyl = (double)j - yg;
+        if constexpr (DEV) {
+            dxl = dxf;
+            dyl = dyf;
+        }
+    }
+    if constexpr (!DEV) {
+        if (chi) {
+            dxl = (double)i - VPLBM_LDG(&bs->q[0]);
+            dyl = (double)j - VPLBM_LDG(&bs->q[1]);
+        }
     }
     return chi;
 }
@@ -647,6 +656,69 @@ __device__ __forceinline__ typename Ln::L mrt_dev_lanes(const StepParams &p, con
     return rho;
 }
 
+// The MRT update in FP64 instructions, for the FP64-storage nodes outside the
+// fixed-point range (fixed64.cuh).  A function of its own: such nodes are
+// rare, and its registers and code stay out of the callers' main path.
+// f: the pulled populations; out: f~; kept: rho, a_x, a_y.
+__device__ __noinline__ void mrt_native_f64(const StepParams &p, const BodyState *__restrict__ bs, bool chi,
+                                            double dxl, double dyl, const double *f, double *out, double *kept)
+{
+    // sums shared by the moments (rows of Eq. 15)
+    const double d13 = f[1] - f[3], d24 = f[2] - f[4], b13 = f[1] + f[3], b24 = f[2] + f[4];
+    const double d56 = f[5] - f[6], d87 = f[8] - f[7], a56 = f[5] + f[6], a78 = f[7] + f[8];
+    const double sx = d56 + d87, ty = a56 - a78, sa = b13 + b24, sd = a56 + a78;
+    const double rho = (f[0] + sa) + sd;
+    const double jx = d13 + sx, jy = d24 + ty;
+    // penalized velocity, Eq. (22) in the eta-stable form
+    const double inv_rho = recip(rho);
+    const double vx = jx * inv_rho + 0.5 * p.gx, vy = jy * inv_rho + 0.5 * p.gy;
+    double ax = 0, ay = 0;
+    if (chi) {
+        ax = -(vx - (bs->v[0] - bs->v[2] * dyl)) * p.pen_k;
+        ay = -(vy - (bs->v[1] + bs->v[2] * dxl)) * p.pen_k;
+    }
+    const double ux = vx + 0.5 * ax, uy = vy + 0.5 * ay;
+    const double Gx = rho * (p.gx + ax), Gy = rho * (p.gy + ay);
+    // moments (rows of Eq. 15); equilibria (Eq. 14); M F closed form;
+    // Eq. (17) with the host-folded factors 1 - s_k and (1 - s_k/2)
+    const double e = fma(-4.0, f[0], fma(2.0, sd, -sa));
+    const double ep = fma(4.0, f[0], fma(-2.0, sa, sd));
+    const double qx = fma(-2.0, d13, sx), qy = fma(-2.0, d24, ty);
+    const double pxx = b13 - b24;
+    const double pxy = (f[5] + f[7]) - (f[6] + f[8]);
+    const auto &k = p.pcd;
+    const double ux2 = ux * ux, uy2 = uy * uy;
+    const double u2r = rho * (ux2 + uy2);
+    const double uG = fma(ux, Gx, uy * Gy);
+    const double e_s = fma(k.om1, e, fma(p.s[1], fma(3.0, u2r, -2.0 * rho), k.h1x6 * uG));
+    const double ep_s = fma(k.om2, ep, fma(p.s[2], fma(-3.0, u2r, rho), k.mh2x6 * uG));
+    const double jx_s = jx + Gx, jy_s = jy + Gy;
+    const double qx_s = fma(k.om4, qx, fma(-p.s[4], rho * ux, k.mh4 * Gx));
+    const double qy_s = fma(k.om6, qy, fma(-p.s[6], rho * uy, k.mh6 * Gy));
+    const double pxx_s = fma(k.om7, pxx, fma(p.s[7], rho * (ux2 - uy2), k.h7x2 * fma(ux, Gx, -uy * Gy)));
+    const double pxy_s = fma(k.om8, pxy, fma(p.s[8], rho * (ux * uy), k.h8 * fma(ux, Gy, uy * Gx)));
+    // back to populations, M^-1 = M^T diag(1/|row|^2)
+    const double r9 = rho * (1.0 / 9.0);
+    const double A = r9 - e_s * (1.0 / 36.0) - ep_s * (1.0 / 18.0);
+    const double B = r9 + e_s * (1.0 / 18.0) + ep_s * (1.0 / 36.0);
+    const double X1 = (jx_s - qx_s) * (1.0 / 6.0), Y1 = (jy_s - qy_s) * (1.0 / 6.0);
+    const double X2 = jx_s * (1.0 / 6.0) + qx_s * (1.0 / 12.0), Y2 = jy_s * (1.0 / 6.0) + qy_s * (1.0 / 12.0);
+    const double Pq = pxx_s * 0.25, Rq = pxy_s * 0.25;
+    out[0] = r9 - e_s * (1.0 / 9.0) + ep_s * (1.0 / 9.0);
+    out[1] = A + X1 + Pq;
+    out[2] = A + Y1 - Pq;
+    out[3] = A - X1 + Pq;
+    out[4] = A - Y1 - Pq;
+    out[5] = B + X2 + Y2 + Rq;
+    out[6] = B - X2 + Y2 - Rq;
+    out[7] = B - X2 - Y2 + Rq;
+    out[8] = B + X2 - Y2 - Rq;
+    if (!(rho > 0.0) || !(rho < 1e30)) *p.err = ERR_NONFINITE;
+    kept[0] = rho;
+    kept[1] = ax;
+    kept[2] = ay;
+}
+
 // The VP-MRT (or BGK) update of one node from its pulled populations f
 // given chi and the lever arm from body_chi: moments, u_s of the body
 // state bs, penalized velocity (Eq. 22), collision with forcing (Eq. 17)
@@ -667,6 +739,39 @@ __device__ __forceinline__ bool node_collide_to(const StepParams &p, const BodyS
         cr = mrt_dev_lanes<Lane1>(p, f, chi, dxl, dyl, bs, store, ax, ay);
         cax = ax;
         cay = ay;
+        return chi;
+    } else if constexpr (COLL == VPLBM_COLLISION_MRT) {
+        // FP64 storage: fixed point where the node is in range
+        if (p.fx.ok) {
+            uint64_t bits[NQ];
+#pragma unroll
+            for (int a = 0; a < NQ; ++a) bits[a] = (uint64_t)__double_as_longlong(f[a]);
+            long long usx = 0, usy = 0, rho = 0, ax = 0, ay = 0;
+            if (chi) {
+                usx = __double2ll_rn((bs->v[0] - bs->v[2] * dyl) * 0x1p61);
+                usy = __double2ll_rn((bs->v[1] + bs->v[2] * dxl) * 0x1p61);
+            }
+            double out[NQ];
+            if (fx_update(p.fx, bits, chi, usx, usy, out, rho, ax, ay)) {
+#pragma unroll
+                for (int a = 0; a < NQ; ++a) store(a, out[a]);
+                if (chi) {   // kept for the solid-node sums
+                    cr = (double)rho * p.fx.unit;
+                    cax = (double)ax * 0x1p-60;
+                    cay = (double)ay * 0x1p-60;
+                }
+                return chi;
+            }
+        }
+        double in[NQ], out[NQ], kept[3];
+#pragma unroll
+        for (int a = 0; a < NQ; ++a) in[a] = f[a];
+        mrt_native_f64(p, bs, chi, dxl, dyl, in, out, kept);
+#pragma unroll
+        for (int a = 0; a < NQ; ++a) store(a, out[a]);
+        cr = kept[0];
+        cax = kept[1];
+        cay = kept[2];
         return chi;
     }
     // sums shared by the moments (rows of Eq. 15)
@@ -741,85 +846,6 @@ __device__ __forceinline__ bool node_collide_to(const StepParams &p, const BodyS
         return chi;
     }
 
-    // moments (rows of Eq. 15); equilibria (Eq. 14); M F closed form;
-    // Eq. (17) with the host-folded factors 1 - s_k and (1 - s_k/2)
-    const T e = fma((T)-4, f[0], fma((T)2, sd, -sa));
-    const T ep = fma((T)4, f[0], fma((T)-2, sa, sd));
-    const T qx = fma((T)-2, d13, sx);
-    const T qy = fma((T)-2, d24, ty);
-    const T pxx = b13 - b24;
-    const T pxy = (f[5] + f[7]) - (f[6] + f[8]);
-
-    const auto &k = folded<T>(p);
-    T e_s, ep_s, A, B, X1, Y1, X2, Y2, Pq, Rq, r9;
-    if constexpr (DEV) {
-        // the same operations with the (x, y) and (e, eps) pairs on the
-        // paired FP32 instructions (each lane rounds like the scalar op)
-        const float2 U = make_float2(ux, uy), G = make_float2(Gx, Gy);
-        const float2 rr = make_float2(rho, rho);
-        const float2 U2 = __fmul2_rn(U, U);
-        const T u2r = rho * (U2.x + U2.y);
-        const T uG = fma(ux, Gx, uy * Gy);
-        const float2 t1 = __ffma2_rn(make_float2(3.f, -3.f), make_float2(u2r, u2r), make_float2(-2.f * rs, rs));
-        const float2 t2 = __fmul2_rn(make_float2(k.h1x6, k.mh2x6), make_float2(uG, uG));
-        const float2 t3 = __ffma2_rn(make_float2(p.sf[1], p.sf[2]), t1, t2);
-        const float2 ES = __ffma2_rn(make_float2(k.om1, k.om2), make_float2(e, ep), t3);
-        e_s = ES.x;
-        ep_s = ES.y;
-        const float2 JS = __fadd2_rn(make_float2(jx, jy), G);
-        const float2 Q = make_float2(qx, qy);
-        const float2 QS = __ffma2_rn(make_float2(k.om4, k.om6), Q,
-                                     __ffma2_rn(make_float2(-p.sf[4], -p.sf[6]), __fmul2_rn(rr, U),
-                                                __fmul2_rn(make_float2(k.mh4, k.mh6), G)));
-        const float2 D = make_float2(U2.x - U2.y, ux * uy);
-        const float2 C = make_float2(fma(ux, Gx, -uy * Gy), fma(ux, Gy, uy * Gx));
-        const float2 PS = __ffma2_rn(make_float2(k.om7, k.om8), make_float2(pxx, pxy),
-                                     __ffma2_rn(make_float2(p.sf[7], p.sf[8]), __fmul2_rn(rr, D),
-                                                __fmul2_rn(make_float2(k.h7x2, k.h8), C)));
-        r9 = rs * (T)(1.0 / 9.0);
-        A = r9 - e_s * (T)(1.0 / 36.0) - ep_s * (T)(1.0 / 18.0);
-        B = r9 + e_s * (T)(1.0 / 18.0) + ep_s * (T)(1.0 / 36.0);
-        const float2 XY1 = __fmul2_rn(__ffma2_rn(QS, make_float2(-1.f, -1.f), JS), make_float2(1.f / 6.f, 1.f / 6.f));
-        const float2 XY2 = __ffma2_rn(QS, make_float2(1.f / 12.f, 1.f / 12.f), __fmul2_rn(JS, make_float2(1.f / 6.f, 1.f / 6.f)));
-        const float2 PR = __fmul2_rn(PS, make_float2(0.25f, 0.25f));
-        X1 = XY1.x; Y1 = XY1.y; X2 = XY2.x; Y2 = XY2.y; Pq = PR.x; Rq = PR.y;
-    } else {
-        const T ux2 = ux * ux, uy2 = uy * uy;
-        const T u2r = rho * (ux2 + uy2);
-        const T uG = fma(ux, Gx, uy * Gy);
-        e_s = fma((T)k.om1, e, fma(par<T>(p.s[1], p.sf[1]), fma((T)3, u2r, (T)-2 * rs), (T)k.h1x6 * uG));
-        ep_s = fma((T)k.om2, ep, fma(par<T>(p.s[2], p.sf[2]), fma((T)-3, u2r, rs), (T)k.mh2x6 * uG));
-        const T jx_s = jx + Gx;
-        const T jy_s = jy + Gy;
-        const T qx_s = fma((T)k.om4, qx, fma(-par<T>(p.s[4], p.sf[4]), rho * ux, (T)k.mh4 * Gx));
-        const T qy_s = fma((T)k.om6, qy, fma(-par<T>(p.s[6], p.sf[6]), rho * uy, (T)k.mh6 * Gy));
-        const T pxx_s = fma((T)k.om7, pxx, fma(par<T>(p.s[7], p.sf[7]), rho * (ux2 - uy2), (T)k.h7x2 * fma(ux, Gx, -uy * Gy)));
-        const T pxy_s = fma((T)k.om8, pxy, fma(par<T>(p.s[8], p.sf[8]), rho * (ux * uy), (T)k.h8 * fma(ux, Gy, uy * Gx)));
-
-        // back to populations, M^-1 = M^T diag(1/|row|^2)
-        r9 = rs * (T)(1.0 / 9.0);
-        A = r9 - e_s * (T)(1.0 / 36.0) - ep_s * (T)(1.0 / 18.0);
-        B = r9 + e_s * (T)(1.0 / 18.0) + ep_s * (T)(1.0 / 36.0);
-        X1 = (jx_s - qx_s) * (T)(1.0 / 6.0);
-        Y1 = (jy_s - qy_s) * (T)(1.0 / 6.0);
-        X2 = jx_s * (T)(1.0 / 6.0) + qx_s * (T)(1.0 / 12.0);
-        Y2 = jy_s * (T)(1.0 / 6.0) + qy_s * (T)(1.0 / 12.0);
-        Pq = pxx_s * (T)0.25;
-        Rq = pxy_s * (T)0.25;
-    }
-
-    store(0, r9 - e_s * (T)(1.0 / 9.0) + ep_s * (T)(1.0 / 9.0));
-    store(1, A + X1 + Pq);
-    store(2, A + Y1 - Pq);
-    store(3, A - X1 + Pq);
-    store(4, A - Y1 - Pq);
-    store(5, B + X2 + Y2 + Rq);
-    store(6, B - X2 + Y2 - Rq);
-    store(7, B - X2 - Y2 + Rq);
-    store(8, B + X2 - Y2 - Rq);
-
-    if (!(rho > (T)0) || !(rho < (T)1e30)) *p.err = ERR_NONFINITE;
-    cr = rho; cax = ax; cay = ay;
     return chi;
 }
 
