@@ -57,6 +57,8 @@ def dominant_kernel(prec: str, launch, kinds: dict) -> str:
         return f"vp_mrt_step_tma<{PREC_ID[prec]}>"
     if launch[0] == "pair":
         return f"vp_mrt_step_pair<{PREC_ID[prec]}, 5, 0>"
+    if launch[0] == "resident":
+        return f"vp_mrt_resident<{PREC_ID[prec]}, 0>"
     # single steps of a two-step choice run the 40-register kernel
     minb = {"scalar": 4, "scalar48": 5, "scalar40": 6, "fused2": 6, "tma": 6}[launch[0]]
     return f"vp_mrt_step<{PREC_ID[prec]}, {minb}, 0, 0>"
@@ -103,10 +105,11 @@ def measured_peak():
 # Sources that make up each step kernel's code: the public header, the
 # internal headers and the translation unit that instantiates it.
 KERNEL_SOURCES = {
-    "vp_mrt_step<": ("vplbm_internal.cuh", "vplbm_node.cuh", "step_scalar.cuh", "step_kernels.cu"),
+    "vp_mrt_step<": ("vplbm_internal.cuh", "fixed64.cuh", "vplbm_node.cuh", "step_scalar.cuh", "step_kernels.cu"),
     "vp_mrt_step2<": ("vplbm_internal.cuh", "vplbm_node.cuh", "step_fused2.cu"),
     "vp_mrt_step_tma<": ("vplbm_internal.cuh", "vplbm_node.cuh", "step_tma.cu"),
     "vp_mrt_step_pair<": ("vplbm_internal.cuh", "vplbm_node.cuh", "step_scalar.cuh", "step_pair.cuh", "step_pair.cu"),
+    "vp_mrt_resident<": ("vplbm_internal.cuh", "fixed64.cuh", "vplbm_node.cuh", "step_resident.cu"),
     "vp_mrt_sweep<": ("vplbm_internal.cuh", "vplbm_node.cuh", "step_scalar.cuh", "step_pair.cuh", "sweep.cu"),
 }
 

@@ -311,12 +311,29 @@ vplbm_status vplbm_get_body_k(vplbm_ctx *ctx, int k, double q[3], double v[3], l
  *                          a lattice edge or near the body take the
  *                          one-node code.  Its populations equal the
  *                          scalar kernel's bit for bit.
+ *  VPLBM_KERNEL_RESIDENT   many time steps per launch, the populations kept
+ *                          in shared memory between them (FP32 or FP64
+ *                          storage, at most one body, a lattice of at most
+ *                          about 530 000 nodes (FP32) or 150 000 (FP64)):
+ *                          what a context of such a lattice does by default
+ *                          and what vplbm_autotune may choose (vplbm_get_launch
+ *                          then names the kernel of its single launches).  One cooperative
+ *                          launch runs up to 4096 steps; it counts as one
+ *                          VPLBM_LAUNCH_ONE_STEP launch.  (block_x,
+ *                          block_y): the blocks of steps that have to be
+ *                          launched one by one (on a stream that is being
+ *                          captured, or where a cooperative launch is
+ *                          refused); 0 x 0 keeps the current ones.  Its
+ *                          populations equal the scalar kernel's bit for
+ *                          bit; its force sums are added in another order.
+ *                          Its first call allocates a workspace of a few MB
+ *                          that the context keeps.
  * Nodes on the lattice edges and near the body always take the same code.
  * The results of different kernels agree to the rounding of the storage
  * precision. */
 typedef enum {
     VPLBM_KERNEL_SCALAR = 0, VPLBM_KERNEL_SCALAR_48 = 1, VPLBM_KERNEL_SCALAR_40 = 2, VPLBM_KERNEL_TMA = 3,
-    VPLBM_KERNEL_FUSED2 = 4, VPLBM_KERNEL_PAIR = 5
+    VPLBM_KERNEL_FUSED2 = 4, VPLBM_KERNEL_PAIR = 5, VPLBM_KERNEL_RESIDENT = 6
 } vplbm_kernel;
 
 /* Kernel and block shape: block_x * block_y threads, block_x a multiple of
@@ -329,12 +346,15 @@ vplbm_status vplbm_get_launch(vplbm_ctx *ctx, int *kernel, int *block_x, int *bl
  * state is saved and restored around the trials) and keep the fastest. */
 vplbm_status vplbm_autotune(vplbm_ctx *ctx, int steps_per_trial);
 
-/* Test hook for the bounded waits of the TMA-staged kernel: when enabled,
+/* Test hook for the bounded waits of the TMA-staged and (when chosen through
+ * vplbm_set_launch) the resident kernel.  Resident: while enabled, its tiles
+ * wait in vain for the pose and give up after 20 ms; the next vplbm_sync
+ * returns VPLBM_ETIMEOUT (initialise or load the state again).  TMA: when enabled,
  * the first shared-memory stage of every block waits for 16 bytes more than
  * its tensor copies deliver, so the wait gives up after about one second,
  * the block leaves once its copies have landed, and the next vplbm_sync
  * returns VPLBM_ETIMEOUT; the context stays usable.  Disable to resume.
- * VPLBM_EUNSUPPORTED unless the TMA-staged kernel is selected. */
+ * VPLBM_EUNSUPPORTED unless one of the two is selected. */
 vplbm_status vplbm_inject_wait_timeout(vplbm_ctx *ctx, int enable);
 
 /* Number of step-kernel launches made by vplbm_step since creation
@@ -345,7 +365,8 @@ vplbm_status vplbm_get_launch_count(vplbm_ctx *ctx, long long *launches);
  * vplbm_get_kernel_launches):
  *  VPLBM_LAUNCH_ONE_STEP   one time step on a scalar step kernel (any
  *                          register budget, shape, or several bodies) or
- *                          on the node-pair kernel;
+ *                          on the node-pair kernel; or one launch of the
+ *                          resident kernel (its steps together);
  *  VPLBM_LAUNCH_TWO_STEP   two time steps on the two-step kernel;
  *  VPLBM_LAUNCH_LOOKAHEAD  the one-thread launch that computes pose n + 1
  *                          of a prescribed path ahead of a run of two-step

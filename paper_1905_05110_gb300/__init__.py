@@ -380,7 +380,8 @@ COLLISIONS = {"mrt": 0, "bgk": 1}
 SHAPES = {"disk": 0, "ellipse": 1, "rectangle": 2}
 BATCH_MODES = {"branches": 0, "tiles": 1, "persistent": 2}
 BATCH_MODE_NAMES = {v: k for k, v in BATCH_MODES.items()}
-KERNELS = {"scalar": 0, "scalar48": 1, "scalar40": 2, "tma": 3, "fused2": 4, "pair": 5}
+KERNELS = {"scalar": 0, "scalar48": 1, "scalar40": 2, "tma": 3, "fused2": 4, "pair": 5,
+           "resident": 6}
 KERNEL_NAMES = {v: k for k, v in KERNELS.items()}
 
 
@@ -650,8 +651,9 @@ class Simulation:
 
     def set_launch(self, kernel, bx=0, by=0):
         """kernel: "scalar" (64-register budget), "scalar48", "scalar40", "tma", "fused2"
-        (two steps per launch; bx, by: the blocks of its single steps) or "pair" (two
-        nodes per thread, FP16 storage) (or its number)."""
+        (two steps per launch; bx, by: the blocks of its single steps), "pair" (two
+        nodes per thread, FP16 storage) or "resident" (many steps per launch of a
+        lattice that fits shared memory) (or its number)."""
         k = KERNELS[kernel] if isinstance(kernel, str) else int(kernel)
         vplbm_set_launch(self.ctx, k, bx, by)
 

@@ -599,9 +599,10 @@ extern "C" vplbm_status vplbm_adjoint(vplbm_ctx *c, const vplbm_adjoint_desc *d,
     // context's scalar step kernel (a TMA-staged choice falls back to the
     // 48-register scalar kernel on 256 x 1 blocks, a two-step choice to its
     // single-step blocks)
-    const bool scalar = c->kernel != KERNEL_TMA;
+    const int rk = step_kernel(c);
+    const bool scalar = rk != KERNEL_TMA;
     const int rbx = scalar ? c->bx : 256, rby = scalar ? c->by : 1;
-    const int rminb = !scalar ? 5 : c->kernel == KERNEL_SCALAR_40 || c->kernel == KERNEL_FUSED2 ? 6 : c->kernel == KERNEL_SCALAR_48 ? 5 : 4;
+    const int rminb = !scalar ? 5 : rk == KERNEL_SCALAR_40 || rk == KERNEL_FUSED2 ? 6 : rk == KERNEL_SCALAR_48 ? 5 : 4;
     int cur = 0;   // lam[cur] holds L_{n+1}, zero-gradient rows [cur] its pending column contributions
     // recompute the states S_{s0} .. S_{s0+len-1} of segment s into store
     // slot set s & 1, on stream sr, straight from one slot to the next (the

@@ -33,7 +33,8 @@ struct vplbm_ctx {
     void *outlet = nullptr;               // convective outlet state, 2 parities x 3 x ny (8-byte slots)
     void *owned = nullptr;                // single allocation when the library owns memory
     long long nstep = 0;
-    int kernel = vplbm::KERNEL_SCALAR;    // KERNEL_SCALAR / _48 / _40 / KERNEL_TMA
+    int kernel = vplbm::KERNEL_SCALAR;    // the launch choice (KERNEL_*)
+    int base_kernel = vplbm::KERNEL_SCALAR;   // under KERNEL_RESIDENT: the kernel of steps that are launched one by one
     int bx = 128, by = 2;
     cudaGraphExec_t graph = nullptr;
     int graph_kernel = -1, graph_bx = -1, graph_by = -1;
@@ -44,6 +45,15 @@ struct vplbm_ctx {
     bool tma_ok = false;
     CUtensorMap tmap[2];
     int tma_grid = 0;
+    // resident kernel: its tiling, and its mailboxes and rings (allocated by
+    // the first resident call, freed by vplbm_destroy)
+    bool res_ok = false;
+    bool res_chosen = false;              // by vplbm_set_launch (not the default)
+    bool res_mute = false;                // test hook
+    vplbm::ResidentPlan res_plan{};
+    void *res_ws = nullptr;
+    size_t res_bytes = 0, res_poses = 0, res_parts = 0;
+    uint32_t res_tag = 1;                 // tag of the next resident step
     // device workspace of vplbm_adjoint (checkpoints, segment stores,
     // adjoint fields, accumulators), kept between calls; grown when a call
     // needs more, freed by vplbm_destroy
@@ -54,6 +64,8 @@ struct vplbm_ctx {
 namespace vplbm {
 // Shared runtime helpers (capi.cu).
 StepParams ctx_params(const vplbm_ctx *c, long long step);        // parameters of step `step`
+inline int step_kernel(const vplbm_ctx *c) { return c->kernel == KERNEL_RESIDENT ? c->base_kernel : c->kernel; }
+void ctx_disable_resident(vplbm_ctx *c);                          // a batch's members step by launches
 cudaError_t ctx_launch(const vplbm_ctx *c, long long step, cudaStream_t stream);
 vplbm_status ctx_read_error(vplbm_ctx *c);                          // latched device errors (syncs)
 vplbm_status report_error(vplbm_status st, const char *msg);

@@ -224,9 +224,10 @@ inline double bounding_radius(const vplbm_body_desc *b)
 }
 
 // Step kernels a context can launch: the scalar kernel with the register
-// budget of 4 / 5 / 6 blocks of 256 threads per SM, the TMA-staged one, and
-// the two-step kernel (two time steps per launch).
-enum { KERNEL_SCALAR = 0, KERNEL_SCALAR_48 = 1, KERNEL_SCALAR_40 = 2, KERNEL_TMA = 3, KERNEL_FUSED2 = 4, KERNEL_PAIR = 5 };
+// budget of 4 / 5 / 6 blocks of 256 threads per SM, the TMA-staged one, the
+// two-step kernel (two time steps per launch), the node-pair kernel and the
+// resident one (many steps per launch).
+enum { KERNEL_SCALAR = 0, KERNEL_SCALAR_48 = 1, KERNEL_SCALAR_40 = 2, KERNEL_TMA = 3, KERNEL_FUSED2 = 4, KERNEL_PAIR = 5, KERNEL_RESIDENT = 6 };
 
 // Node-pair kernel (step_pair.cu): FP16 storage, MRT, one body, even nx;
 // blocks of bx x by threads on tiles of 2 bx x by nodes (the body blocks on
@@ -301,6 +302,38 @@ int sweep_supported(int precision, int collision);
 cudaError_t sweep_max_grid(int precision, bool disk, bool psmem, int bx, int by, int *grid);
 cudaError_t launch_sweep(int precision, bool disk, bool psmem, const SweepLaunch &sl, int grid, int bx, int by,
                          cudaStream_t stream);
+
+// Resident kernel (step_resident.cu): many steps of a small lattice in one
+// cooperative launch of tiles + 1 blocks, the populations in shared memory.
+constexpr int RES_PART_RING = 16;      // steps of partial sums in flight (a tile is at most 8 steps ahead of the tail)
+constexpr int RES_MAX_STEPS = 4096;    // steps of one launch at most (a few milliseconds)
+struct ResidentPlan {
+    int ntx, nty, tiles;   // tile columns and rows (tiles of nx / ntx x ny / nty nodes, rounded up or down)
+    int mw, mh;            // largest tile width and height
+    int k;                 // nodes per thread
+    int items;             // mailbox values per tile and parity
+    int part_slots;        // tiles a body can meet at most
+    int part_copies;       // of the forces: 1, or 1 + part_slots (a free body)
+    int pose_ring;         // poses in flight: more than the steps a tile can lag behind the tail
+    int edge_at, smem;     // start of the edge tables in the dynamic shared memory, its size
+};
+struct ResidentLaunch {
+    StepParams p;          // of the first step: fin, bs_in, conv_in
+    ResidentPlan t;
+    void *fout;            // the state after the last step
+    BodyState *bs_out;
+    void *conv_out;
+    uint64_t *mail, *poses, *parts;   // tagged words (resident_bytes)
+    double rk[3][4];       // a free body's step as an affine map, per degree of freedom (resident_rk)
+    uint32_t tag0;         // tag of the first step; tags of earlier launches are below it, 0 is never used
+    int nsteps;
+    unsigned long long timeout_ns;
+    int mute;              // test hook: the tail publishes nothing
+};
+int resident_k(int precision, int w, int h, int *edge_at, int *smem);
+size_t resident_bytes(const ResidentPlan &t, int precision, size_t *poses, size_t *parts);
+void resident_rk(const DevBody &b, double rk[3][4]);
+cudaError_t launch_resident(int precision, const ResidentLaunch &L, cudaStream_t stream);
 
 // Launchers (step_kernels.cu).  All are asynchronous on `stream`.
 cudaError_t launch_step(int precision, const StepParams &p, int bx, int by, cudaStream_t stream, int minb = 4);

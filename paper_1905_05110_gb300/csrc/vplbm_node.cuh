@@ -32,8 +32,11 @@ template <int P> constexpr int budget_blocks(int minb) { return P != VPLBM_F64 |
 // several steps in one launch reads data it wrote itself after a grid-wide
 // barrier, which the non-coherent path may serve stale: its translation unit
 // defines VPLBM_COHERENT_LOADS before including this header, and its loads
-// go to L2 (ld.global.cg).
-#ifdef VPLBM_COHERENT_LOADS
+// go to L2 (ld.global.cg).  One that keeps them in shared memory defines
+// VPLBM_PLAIN_LOADS.
+#if defined(VPLBM_PLAIN_LOADS)
+#define VPLBM_LDG(ptr) (*(ptr))
+#elif defined(VPLBM_COHERENT_LOADS)
 #define VPLBM_LDG(ptr) __ldcg(ptr)
 #else
 #define VPLBM_LDG(ptr) __ldg(ptr)
@@ -318,6 +321,8 @@ __device__ __forceinline__ float2 ff_add(float2 a, float2 b)
 
 template <int P> struct SumT { using A = float2; using V = float; };
 template <> struct SumT<VPLBM_F64> { using A = double; using V = double; };
+template <typename A> struct SumVal { using V = float; };
+template <> struct SumVal<double> { using V = double; };
 
 __device__ __forceinline__ void acc_add(double &a, double b) { a += b; }
 __device__ __forceinline__ void acc_add(float2 &a, float2 b) { a = ff_add(a, b); }
@@ -328,6 +333,11 @@ __device__ __forceinline__ double acc_shfl_down(double a, int off) { return __sh
 __device__ __forceinline__ float2 acc_shfl_down(float2 a, int off)
 {
     return make_float2(__shfl_down_sync(0xffffffffu, a.x, off), __shfl_down_sync(0xffffffffu, a.y, off));
+}
+__device__ __forceinline__ double acc_shfl(double a, int lane) { return __shfl_sync(0xffffffffu, a, lane); }
+__device__ __forceinline__ float2 acc_shfl(float2 a, int lane)
+{
+    return make_float2(__shfl_sync(0xffffffffu, a.x, lane), __shfl_sync(0xffffffffu, a.y, lane));
 }
 __device__ __forceinline__ double acc_value(double a) { return a; }
 __device__ __forceinline__ double acc_value(float2 a) { return (double)a.x + (double)a.y; }   // exact
@@ -583,10 +593,12 @@ struct Lane2 {
 // a = 0 off the body: u = j / rho + g / 2), stored through store(a, value).
 // Returns rho.  Lane1 only: chi and the lever arm (dxl, dyl) of the node,
 // and (ax, ay) = a for the solid-node sums.
-template <class Ln, class Store>
-__device__ __forceinline__ typename Ln::L mrt_dev_lanes(const StepParams &p, const typename Ln::L f[NQ], bool chi,
-                                                        float dxl, float dyl, const BodyState *__restrict__ bs,
-                                                        const Store &store, float &ax_out, float &ay_out)
+// mrt_dev_core: the same with the forcing of the node(s) given as a function
+// force(rho, ux, uy, Gx, Gy) that turns the unpenalized velocity and G = rho g
+// into the penalized ones.
+template <class Ln, class Force, class Store>
+__device__ __forceinline__ typename Ln::L mrt_dev_core(const StepParams &p, const typename Ln::L f[NQ],
+                                                       const Force &force, const Store &store)
 {
     using L = typename Ln::L;
     const L d13 = Ln::sub(f[1], f[3]), d24 = Ln::sub(f[2], f[4]), b13 = Ln::add(f[1], f[3]), b24 = Ln::add(f[2], f[4]);
@@ -598,21 +610,7 @@ __device__ __forceinline__ typename Ln::L mrt_dev_lanes(const StepParams &p, con
     const L inv_rho = Ln::recip(rho);
     L ux = Ln::fma(jx, inv_rho, Ln::c(p.pc.hgx)), uy = Ln::fma(jy, inv_rho, Ln::c(p.pc.hgy));
     L Gx = Ln::mul(rho, Ln::c(p.gxf)), Gy = Ln::mul(rho, Ln::c(p.gyf));
-    ax_out = 0.f;
-    ay_out = 0.f;
-    if constexpr (Ln::SCALAR) {
-        if (chi) {   // Eq. (22), eta-stable form: a = (u_s - v) / (eta + 1/2), u = v + a / 2
-            const float4 vv = VPLBM_LDG(reinterpret_cast<const float4 *>(&bs->vxf));
-            const float usx = __fmaf_rn(-vv.z, dyl, vv.x), usy = __fmaf_rn(vv.z, dxl, vv.y);
-            const float ax = __fmul_rn(__fsub_rn(usx, ux), p.pen_kf), ay = __fmul_rn(__fsub_rn(usy, uy), p.pen_kf);
-            Gx = __fmul_rn(rho, __fadd_rn(p.gxf, ax));
-            Gy = __fmul_rn(rho, __fadd_rn(p.gyf, ay));
-            ux = __fmaf_rn(0.5f, ax, ux);
-            uy = __fmaf_rn(0.5f, ay, uy);
-            ax_out = ax;
-            ay_out = ay;
-        }
-    }
+    force(rho, ux, uy, Gx, Gy);
     const auto &k = p.pc;
     const L e = Ln::fma(Ln::c(-4.f), f[0], Ln::fms(Ln::c(2.f), sd, sa));
     const L ep = Ln::fma(Ln::c(4.f), f[0], Ln::fma(Ln::c(-2.f), sa, sd));
@@ -654,6 +652,56 @@ __device__ __forceinline__ typename Ln::L mrt_dev_lanes(const StepParams &p, con
     store(8, Ln::sub(Ln::sub(Ln::add(B, X2), Y2), Rq));
     if (Ln::bad(rho)) *p.err = ERR_NONFINITE;
     return rho;
+}
+
+template <class Ln, class Store>
+__device__ __forceinline__ typename Ln::L mrt_dev_lanes(const StepParams &p, const typename Ln::L f[NQ], bool chi,
+                                                        float dxl, float dyl, const BodyState *__restrict__ bs,
+                                                        const Store &store, float &ax_out, float &ay_out)
+{
+    using L = typename Ln::L;
+    ax_out = 0.f;
+    ay_out = 0.f;
+    auto force = [&](const L &rho, L &ux, L &uy, L &Gx, L &Gy) {
+        if constexpr (Ln::SCALAR) {
+            if (chi) {   // Eq. (22), eta-stable form: a = (u_s - v) / (eta + 1/2), u = v + a / 2
+                const float4 vv = VPLBM_LDG(reinterpret_cast<const float4 *>(&bs->vxf));
+                const float usx = __fmaf_rn(-vv.z, dyl, vv.x), usy = __fmaf_rn(vv.z, dxl, vv.y);
+                const float ax = __fmul_rn(__fsub_rn(usx, ux), p.pen_kf), ay = __fmul_rn(__fsub_rn(usy, uy), p.pen_kf);
+                Gx = __fmul_rn(rho, __fadd_rn(p.gxf, ax));
+                Gy = __fmul_rn(rho, __fadd_rn(p.gyf, ay));
+                ux = __fmaf_rn(0.5f, ax, ux);
+                uy = __fmaf_rn(0.5f, ay, uy);
+                ax_out = ax;
+                ay_out = ay;
+            }
+        }
+    };
+    return mrt_dev_core<Ln>(p, f, force, store);
+}
+
+// Two nodes on paired lanes, either or both of them solid (chi0, chi1; lever
+// arms in the lanes of dx, dy): every lane the operations of the one-node
+// form.  (ax, ay) of a lane is kept where it is solid.
+template <class Store>
+__device__ __forceinline__ float2 mrt_dev_pair_chi(const StepParams &p, const float2 f[NQ], bool chi0, bool chi1,
+                                                   float2 dx, float2 dy, const BodyState *__restrict__ bs,
+                                                   const Store &store, float2 &ax_out, float2 &ay_out)
+{
+    using Ln = Lane2;
+    auto sel = [&](float2 a, float2 b) { return make_float2(chi0 ? a.x : b.x, chi1 ? a.y : b.y); };
+    auto force = [&](const float2 &rho, float2 &ux, float2 &uy, float2 &Gx, float2 &Gy) {
+        const float4 vv = VPLBM_LDG(reinterpret_cast<const float4 *>(&bs->vxf));
+        const float2 usx = Ln::fma(Ln::c(-vv.z), dy, Ln::c(vv.x)), usy = Ln::fma(Ln::c(vv.z), dx, Ln::c(vv.y));
+        const float2 ax = Ln::mul(Ln::sub(usx, ux), Ln::c(p.pen_kf)), ay = Ln::mul(Ln::sub(usy, uy), Ln::c(p.pen_kf));
+        Gx = sel(Ln::mul(rho, Ln::add(Ln::c(p.gxf), ax)), Gx);
+        Gy = sel(Ln::mul(rho, Ln::add(Ln::c(p.gyf), ay)), Gy);
+        ux = sel(Ln::fma(Ln::c(0.5f), ax, ux), ux);
+        uy = sel(Ln::fma(Ln::c(0.5f), ay, uy), uy);
+        ax_out = ax;
+        ay_out = ay;
+    };
+    return mrt_dev_core<Ln>(p, f, force, store);
 }
 
 // The MRT update in FP64 instructions, for the FP64-storage nodes outside the
