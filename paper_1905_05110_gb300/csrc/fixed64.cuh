@@ -63,6 +63,8 @@ struct FixedConsts {
     FxFactor h1, h2, h4, h6, h7, h8, sixth, k4;
     long long gvx, gvy;         // g 2^60
     int forced;                 // g is not zero
+    long long rho0;             // in units of 2^(E - 59)
+    FxFactor w0, w1, w2;        // the weights
 };
 
 inline FxFactor fx_factor(double r)
@@ -96,6 +98,8 @@ inline void fold_fixed(FixedConsts &k, const double *s, double rho0, double gx, 
     k.gvx = llrint(ldexp(gx, 60));
     k.gvy = llrint(ldexp(gy, 60));
     k.forced = gx != 0.0 || gy != 0.0;
+    k.rho0 = llrint(ldexp(rho0, 59 - e));
+    k.w0 = fx_factor(4.0 / 9.0); k.w1 = fx_factor(1.0 / 9.0); k.w2 = fx_factor(1.0 / 36.0);
 }
 
 VPLBM_FX int fx_clz(uint32_t x)
@@ -126,6 +130,30 @@ VPLBM_FX double fx_double(uint64_t b)
     double d;
     memcpy(&d, &b, 8);
     return d;
+#endif
+}
+
+VPLBM_FX uint32_t fx_float_bits(float f)
+{
+#if defined(__CUDA_ARCH__)
+    return __float_as_uint(f);
+#else
+    uint32_t b;
+    memcpy(&b, &f, 4);
+    return b;
+#endif
+}
+
+// 2^k, -126 <= k <= 127.
+VPLBM_FX float fx_pow2f(int k)
+{
+    const uint32_t b = (uint32_t)(127 + k) << 23;
+#if defined(__CUDA_ARCH__)
+    return __uint_as_float(b);
+#else
+    float f;
+    memcpy(&f, &b, 4);
+    return f;
 #endif
 }
 
@@ -337,6 +365,145 @@ bool fx_update(const FixedConsts &k, const uint64_t fb[9], bool chi, long long u
 #endif
     for (int a = 0; a < 9; ++a) out[a] = fx_to(f[a], k.e);
     rho_o = rho;
+    return true;
+}
+
+// ---- fields and equilibria ------------------------------------------------
+
+// x 2^k as a double, to nearest even, for any x.
+VPLBM_FX double fx_signed_to(long long x, int k)
+{
+    if (x == 0) return 0.0;
+    const uint64_t sign = (uint64_t)x & 0x8000000000000000ull, m = x < 0 ? 0 - (uint64_t)x : (uint64_t)x;
+    const uint32_t hi = (uint32_t)(m >> 32);
+    const int n = hi ? fx_clz(hi) : 32 + fx_clz((uint32_t)m);
+    const uint64_t y = m << n;   // leading bit at 63
+    const uint64_t q = y >> 11, half = (y >> 10) & 1, rest = (y & 0x3ff) | (q & 1);
+    return fx_double(sign | ((q + (half & (rest != 0))) + ((uint64_t)(1023 + 63 - 1 + k - n) << 52)));
+}
+
+// x 2^k as a float, to nearest even, for |x| < 2^62 and a result in the
+// normal range (or zero).
+VPLBM_FX float fx_signed_to_float(long long x, int k)
+{
+    const uint64_t m = x < 0 ? 0 - (uint64_t)x : (uint64_t)x;
+    const uint32_t hi = (uint32_t)(m >> 32);
+    const int n = hi ? fx_clz(hi) : 32 + fx_clz((uint32_t)m | 1u);
+    const uint64_t y = m << n;
+    const uint32_t t = (uint32_t)(y >> 32) | ((uint32_t)y != 0);   // the leading 32 bits, the rest sticky
+    const float f = (float)t * fx_pow2f(k + 32 - n);
+    return x < 0 ? -f : f;
+}
+
+// A float of magnitude below 2^(E - 3) in units of 2^(E - 62) (truncated).
+VPLBM_FX long long fx_from_float(uint32_t b, int e)
+{
+    const uint32_t m = (b & 0x7fffffu) | 0x800000u, ex = (b >> 23) & 0xffu;
+    const uint32_t s = (uint32_t)(123 + e) - ex;
+    const uint64_t x = ((uint64_t)m << 35) >> (s < 63 ? s : 63);
+    return (b >> 31) ? -(long long)x : (long long)x;
+}
+
+// A double of magnitude below 1/4 times 2^61 (truncated).
+VPLBM_FX long long fx_from_signed(uint64_t b)
+{
+    const uint64_t m = ((b & 0xfffffffffffffull) | (1ull << 52)) << 10;
+    const uint32_t s = 1024u - (uint32_t)((b >> 52) & 0x7ff);
+    const uint64_t x = s < 64 ? m >> s : 0;
+    return (long long)b < 0 ? -(long long)x : (long long)x;
+}
+
+// rho and u of nine pulled populations away from the body, without a uniform
+// acceleration: FP64 storage, and FP32 / FP16 storage (deviations, as floats).
+// False if the node is out of range.
+VPLBM_FX bool fx_moments(const FixedConsts &k, const uint64_t fb[9], double &rho_o, double &ux_o, double &uy_o)
+{
+    uint32_t top = 0, low = 0xffffffffu;
+    long long f[9];
+#if defined(__CUDA_ARCH__)
+#pragma unroll
+#endif
+    for (int a = 0; a < 9; ++a) {
+        const uint32_t hi = (uint32_t)(fb[a] >> 32);
+        top = hi > top ? hi : top;
+        low = hi < low ? hi : low;
+        f[a] = fx_from(fb[a], k.e);
+    }
+    if (top >= k.hi_max || low < k.hi_min) return false;
+    const long long sx = f[5] - f[6] - f[7] + f[8], sy = f[5] + f[6] - f[7] - f[8];
+    const long long rho = f[0] + f[1] + f[2] + f[3] + f[4] + f[5] + f[6] + f[7] + f[8];
+    const long long jx = f[1] - f[3] + sx, jy = f[2] - f[4] + sy;
+    constexpr long long J = 201769274521386496LL;   // 0.35 2^59
+    if ((uint64_t)(rho - (1LL << 58)) >= (uint64_t)(1LL << 59) || (uint64_t)(jx + J) >= (uint64_t)(2 * J) ||
+        (uint64_t)(jy + J) >= (uint64_t)(2 * J))
+        return false;
+    const FxFactor inv = fx_split(fx_recip(rho));
+    rho_o = fx_to(rho, k.e);
+    ux_o = fx_signed_to(fx_mul((long long)((uint64_t)jx << 5), inv), -61);
+    uy_o = fx_signed_to(fx_mul((long long)((uint64_t)jy << 5), inv), -61);
+    return true;
+}
+
+VPLBM_FX bool fx_moments_dev(const FixedConsts &k, const float d[9], double &rho_o, double &ux_o, double &uy_o)
+{
+    uint32_t top = 0;
+    long long f[9];
+#if defined(__CUDA_ARCH__)
+#pragma unroll
+#endif
+    for (int a = 0; a < 9; ++a) {
+        const uint32_t b = fx_float_bits(d[a]), m = b & 0x7fffffffu;
+        top = m > top ? m : top;
+        f[a] = fx_from_float(b, k.e);
+    }
+    if (k.e < -30 || k.e > 60 || top >= (uint32_t)(124 + k.e) << 23) return false;
+    const long long sx = f[5] - f[6] - f[7] + f[8], sy = f[5] + f[6] - f[7] - f[8];
+    const long long rs = f[0] + f[1] + f[2] + f[3] + f[4] + f[5] + f[6] + f[7] + f[8];
+    const long long jx = f[1] - f[3] + sx, jy = f[2] - f[4] + sy;
+    const long long rho = k.rho0 + ((rs + 4) >> 3);
+    constexpr long long J = 1LL << 59;   // |j| < 1/8: j << 3 below stays in 62 bits
+    if ((uint64_t)(rho - (1LL << 58)) >= (uint64_t)(1LL << 59) || (uint64_t)(jx + J) >= (uint64_t)(2 * J) ||
+        (uint64_t)(jy + J) >= (uint64_t)(2 * J))
+        return false;
+    const FxFactor inv = fx_split(fx_recip(rho));   // 2^120 / rho
+    rho_o = fx_to(rho, k.e);
+    ux_o = fx_signed_to(fx_mul((long long)((uint64_t)jx << 3), inv), -62);
+    uy_o = fx_signed_to(fx_mul((long long)((uint64_t)jy << 3), inv), -62);
+    return true;
+}
+
+// Equilibrium (Eq. 11) of (rho, u): val[a] in units of 2^(E - 62) for the
+// deviation f_a - w_a rho0 (dev), of 2^(E - 59) for the full f_a.  False if
+// out of range (|u| >= 1/4, rho outside [rho0 / 2, 1.5 2^E); dev: a density
+// further than 2^(E - 4) from rho0).
+VPLBM_FX bool fx_equilibrium(const FixedConsts &k, uint64_t rho_b, uint64_t ux_b, uint64_t uy_b, bool dev, long long val[9])
+{
+    const uint32_t rh = (uint32_t)(rho_b >> 32), xh = (uint32_t)(ux_b >> 32) & 0x7fffffffu, yh = (uint32_t)(uy_b >> 32) & 0x7fffffffu;
+    // rho in [2^(E-1), 2^(E+1)): twice the range of a population, so on the
+    // grid as twice the value of its half
+    if (dev && (k.e < -30 || k.e > 60)) return false;
+    if (rh < (unsigned)(1022 + k.e) << 20 || rh >= (unsigned)(1024 + k.e) << 20 || xh >= 0x3fd00000u || yh >= 0x3fd00000u) return false;
+    const long long rho = 2 * fx_from(rho_b - (1ull << 52), k.e);
+    if (rho >= (3LL << 58)) return false;
+    const long long ux = fx_from_signed(ux_b), uy = fx_from_signed(uy_b);   // 2^61
+    const FxFactor fx = fx_split(ux), fy = fx_split(uy);
+    const long long xx = fx_mul(ux, fx), yy = fx_mul(uy, fy), xy = fx_mul(ux, fy);   // 2^58
+    const long long drho = rho - k.rho0;
+    if (dev && (uint64_t)(drho + (1LL << 55)) >= (uint64_t)(1LL << 56)) return false;
+    const long long r8 = (long long)((uint64_t)rho << 3);
+    const long long u15 = 6 * (xx + yy);   // 3/2 u^2 2^60
+#if defined(__CUDA_ARCH__)
+#pragma unroll
+#endif
+    for (int a = 0; a < 9; ++a) {
+        const int cx = a == 1 || a == 5 || a == 8 ? 1 : (a == 3 || a == 6 || a == 7 ? -1 : 0);
+        const int cy = a == 2 || a == 5 || a == 6 ? 1 : (a == 4 || a == 7 || a == 8 ? -1 : 0);
+        const long long cu = cx * ux + cy * uy, cu2 = (cx ? xx : 0) + (cy ? yy : 0) + 2 * cx * cy * xy;
+        const long long poly = ((3 * cu) >> 1) + 18 * cu2 - u15;   // 3 c.u + 9/2 (c.u)^2 - 3/2 u^2, 2^60
+        const long long rp = fx_mul(r8, fx_split(2 * poly));        // rho poly, 2^(E - 59)
+        const FxFactor w = a == 0 ? k.w0 : a <= 4 ? k.w1 : k.w2;    // w_a / 2^0, 4/9 < 1/2
+        val[a] = dev ? fx_mul((drho + rp) * 8, w) : fx_mul(rho + rp, w);
+    }
     return true;
 }
 

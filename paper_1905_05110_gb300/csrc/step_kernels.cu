@@ -64,6 +64,12 @@ __global__ void __launch_bounds__(256, P == VPLBM_F64 ? 4 : 5) vp_mrt_step_batch
 }
 
 // ---- equilibrium initialisation (Eq. 11) -------------------------------
+//
+// In fixed point (fixed64.cuh) where the node is in range: 80 FP64
+// instructions a node made this kernel six times as long as its memory
+// traffic on GB300 (2048 x 1024, FP32 storage, us per call: uniform state 312 ->
+// 75, fields read from page-locked host memory 359 -> 297, of which the 50 MB
+// over the CPU-GPU link take 243).
 
 template <int P>
 __global__ void init_equilibrium_kernel(const StepParams p, const double *rho_f, const double *ux_f, const double *uy_f)
@@ -76,16 +82,26 @@ __global__ void init_equilibrium_kernel(const StepParams p, const double *rho_f,
     const double rho = rho_f ? rho_f[k] : p.rho0;
     const double ux = ux_f ? ux_f[k] : 0.0;
     const double uy = uy_f ? uy_f[k] : 0.0;
-    const double u2 = ux * ux + uy * uy;
     S *fout = static_cast<S *>(p.fout);
+    long long val[NQ];
+    if (p.fx.ok && fx_equilibrium(p.fx, (uint64_t)__double_as_longlong(rho), (uint64_t)__double_as_longlong(ux),
+                                  (uint64_t)__double_as_longlong(uy), Prec<P>::DEV, val)) {
+#pragma unroll
+        for (int a = 0; a < NQ; ++a) {
+            if constexpr (Prec<P>::DEV) stv(fout + a * p.ps + k, fx_signed_to_float(val[a], p.fx.e - 62));
+            else stv(fout + a * p.ps + k, fx_signed_to(val[a], p.fx.e - 59));
+        }
+        return;
+    }
+    const double u2 = ux * ux + uy * uy;
 #pragma unroll
     for (int a = 0; a < NQ; ++a) {
         const double cu = cx_of(a) * ux + cy_of(a) * uy;
         const double poly = 3.0 * cu + 4.5 * cu * cu - 1.5 * u2;
-        double val;
-        if (Prec<P>::DEV) val = w_of(a) * ((rho - p.rho0) + rho * poly);
-        else val = w_of(a) * rho * (1.0 + poly);
-        stv(fout + a * p.ps + k, (typename Prec<P>::T)val);
+        double v;
+        if (Prec<P>::DEV) v = w_of(a) * ((rho - p.rho0) + rho * poly);
+        else v = w_of(a) * rho * (1.0 + poly);
+        stv(fout + a * p.ps + k, (typename Prec<P>::T)v);
     }
 }
 
@@ -107,6 +123,11 @@ __global__ void outlet_reset_kernel(const StepParams p)
 }
 
 // ---- macroscopic fields of the current step (Eqs. 19-22) ---------------
+//
+// Away from the bodies in fixed point where the node is in range, for the
+// same reason (60 FP64 instructions a node; 2048 x 1024, FP32 storage:
+// us per call to the device 299 -> 41, to page-locked host memory 351 -> 312,
+// of which the link takes 263).
 
 template <int P>
 __global__ void fields_kernel(const StepParams p, double *rho_o, double *ux_o, double *uy_o)
@@ -119,6 +140,31 @@ __global__ void fields_kernel(const StepParams p, double *rho_o, double *ux_o, d
     const S *fin = static_cast<const S *>(p.fin);
     T f[NQ];
     pull_all<P>(p, fin, i, j, f);
+    const long long k = (long long)j * p.nx + i;
+    // the nodes that may be solid (derive_pose's range): chi is tested there
+    bool near = false;
+    for (int m = 0; m < (p.nbodies > 1 ? p.nbodies : 1); ++m) {
+        const int4 r = *reinterpret_cast<const int4 *>(&p.bs_in[m].ilo);   // ilo, ihi, jlo, jhi
+        near = near || (i >= r.x && i <= r.y && j >= r.z && j <= r.w);
+    }
+    if (!near && p.fx.ok && !p.fx.forced) {
+        double rho, ux, uy;
+        bool done;
+        if constexpr (Prec<P>::DEV) {
+            done = fx_moments_dev(p.fx, f, rho, ux, uy);
+        } else {
+            uint64_t bits[NQ];
+#pragma unroll
+            for (int a = 0; a < NQ; ++a) bits[a] = (uint64_t)__double_as_longlong(f[a]);
+            done = fx_moments(p.fx, bits, rho, ux, uy);
+        }
+        if (done) {
+            if (rho_o) rho_o[k] = rho;
+            if (ux_o) ux_o[k] = ux;
+            if (uy_o) uy_o[k] = uy;
+            return;
+        }
+    }
     double rs = 0, jx = 0, jy = 0;
 #pragma unroll
     for (int a = 0; a < NQ; ++a) {
@@ -151,7 +197,6 @@ __global__ void fields_kernel(const StepParams p, double *rho_o, double *ux_o, d
         ax = -(vx - usx) / (p.eta + 0.5);
         ay = -(vy - usy) / (p.eta + 0.5);
     }
-    const long long k = (long long)j * p.nx + i;
     if (rho_o) rho_o[k] = rho;
     if (ux_o) ux_o[k] = vx + 0.5 * ax;
     if (uy_o) uy_o[k] = vy + 0.5 * ay;
