@@ -241,12 +241,7 @@ struct FxForced {
     long long de, dep, dqx, dqy, dp, dr, gx6, gy6, ax, ay;                   // out
 };
 
-#if defined(__CUDACC__)
-__device__ __noinline__
-#else
-inline
-#endif
-bool fx_forced(const FixedConsts &k, bool chi, FxForced &w)
+VPLBM_FX bool fx_forced_here(const FixedConsts &k, bool chi, FxForced &w)
 {
     const long long wx = w.vx + k.gvx, wy = w.vy + k.gvy;   // v = j / rho + g / 2
     long long ax = 0, ay = 0;                               // a 2^60
@@ -279,10 +274,19 @@ bool fx_forced(const FixedConsts &k, bool chi, FxForced &w)
     return true;
 }
 
+#if defined(__CUDACC__)
+__device__ __noinline__
+#else
+inline
+#endif
+bool fx_forced(const FixedConsts &k, bool chi, FxForced &w) { return fx_forced_here(k, chi, w); }
+
 // One node: pulled populations f (bits of doubles) -> post-collision
 // populations out.  chi: the node is in a body of solid velocity us (times
 // 2^61).  Returns false (out untouched) if the node is out of range; rho and
 // a 2^60 (the penalization's acceleration) are kept for the body's sums.
+// HERE: a caller of solid nodes only has the penalized part inlined.
+template <bool HERE = false>
 #if defined(__CUDACC__)
 __device__ __forceinline__
 #else
@@ -320,7 +324,7 @@ bool fx_update(const FixedConsts &k, const uint64_t fb[9], bool chi, long long u
         FxForced w;
         w.rho = rho; w.jx = jx; w.jy = jy; w.vx = vx; w.vy = vy; w.usx = usx; w.usy = usy;
         w.f0 = f[0]; w.sa = sa; w.sd = sd; w.qx = dqx; w.qy = dqy; w.pxx = b13 - b24; w.pxy = d56 - d87;
-        if (!fx_forced(k, chi, w)) return false;
+        if (!(HERE ? fx_forced_here(k, chi, w) : fx_forced(k, chi, w))) return false;
         de = w.de; dep = w.dep; dqx = w.dqx; dqy = w.dqy; dp = w.dp; dr = w.dr;
         gx6 = w.gx6; gy6 = w.gy6;
         ax_o = w.ax;
@@ -382,14 +386,19 @@ VPLBM_FX double fx_signed_to(long long x, int k)
     return fx_double(sign | ((q + (half & (rest != 0))) + ((uint64_t)(1023 + 63 - 1 + k - n) << 52)));
 }
 
-// x 2^k as a float, to nearest even, for |x| < 2^62 and a result in the
-// normal range (or zero).
-VPLBM_FX float fx_signed_to_float(long long x, int k)
+// x 2^k as a float, to nearest, for |x| < 2^62 and a result in the normal
+// range (or zero).  near_tie is set where x is within 512 units of halfway
+// between two floats: FP64 arithmetic, whose error is below that, could round
+// the other way there.
+VPLBM_FX float fx_signed_to_float(long long x, int k, bool &near_tie)
 {
+    if (x == 0) return 0.f;
     const uint64_t m = x < 0 ? 0 - (uint64_t)x : (uint64_t)x;
     const uint32_t hi = (uint32_t)(m >> 32);
-    const int n = hi ? fx_clz(hi) : 32 + fx_clz((uint32_t)m | 1u);
+    const int n = hi ? fx_clz(hi) : 32 + fx_clz((uint32_t)m);
     const uint64_t y = m << n;
+    const long long off = (long long)(y & 0xffffffffffull) - (1LL << 39);   // from halfway
+    near_tie = near_tie || n >= 30 || (off < 0 ? -off : off) <= (512LL << n);
     const uint32_t t = (uint32_t)(y >> 32) | ((uint32_t)y != 0);   // the leading 32 bits, the rest sticky
     const float f = (float)t * fx_pow2f(k + 32 - n);
     return x < 0 ? -f : f;
@@ -404,12 +413,14 @@ VPLBM_FX long long fx_from_float(uint32_t b, int e)
     return (b >> 31) ? -(long long)x : (long long)x;
 }
 
-// A double of magnitude below 1/4 times 2^61 (truncated).
+// A double of magnitude below 1/4 times 2^61, to nearest even.
 VPLBM_FX long long fx_from_signed(uint64_t b)
 {
     const uint64_t m = ((b & 0xfffffffffffffull) | (1ull << 52)) << 10;
-    const uint32_t s = 1024u - (uint32_t)((b >> 52) & 0x7ff);
-    const uint64_t x = s < 64 ? m >> s : 0;
+    const uint32_t s = 1024u - (uint32_t)((b >> 52) & 0x7ff);   // 3 or more
+    if (s > 63) return 0;
+    const uint64_t q = m >> s, half = (m >> (s - 1)) & 1, rest = (m << (65 - s)) | (q & 1);
+    const uint64_t x = q + (half & (rest != 0));
     return (long long)b < 0 ? -(long long)x : (long long)x;
 }
 

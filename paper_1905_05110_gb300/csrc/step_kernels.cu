@@ -86,12 +86,20 @@ __global__ void init_equilibrium_kernel(const StepParams p, const double *rho_f,
     long long val[NQ];
     if (p.fx.ok && fx_equilibrium(p.fx, (uint64_t)__double_as_longlong(rho), (uint64_t)__double_as_longlong(ux),
                                   (uint64_t)__double_as_longlong(uy), Prec<P>::DEV, val)) {
+        // FP32 and FP16 storage: the populations that the FP64 code below
+        // stores, so a node with one near a rounding boundary is left to it
+        bool near_tie = false;
+        typename Prec<P>::T v[NQ];
 #pragma unroll
         for (int a = 0; a < NQ; ++a) {
-            if constexpr (Prec<P>::DEV) stv(fout + a * p.ps + k, fx_signed_to_float(val[a], p.fx.e - 62));
-            else stv(fout + a * p.ps + k, fx_signed_to(val[a], p.fx.e - 59));
+            if constexpr (Prec<P>::DEV) v[a] = fx_signed_to_float(val[a], p.fx.e - 62, near_tie);
+            else v[a] = fx_signed_to(val[a], p.fx.e - 59);
         }
-        return;
+        if (!near_tie) {
+#pragma unroll
+            for (int a = 0; a < NQ; ++a) stv(fout + a * p.ps + k, v[a]);
+            return;
+        }
     }
     const double u2 = ux * ux + uy * uy;
 #pragma unroll

@@ -103,7 +103,6 @@ struct StepParams {
     float rho0f, gxf, gyf, pen_kf, r2f;
     FoldedConsts<float> pc;       // FP32 folded factors
     FoldedConsts<double> pcd;     // FP64 folded factors
-    FixedConsts fx;               // the FP64 kernel's fixed-point constants
     int bc[4];
     double wall_u0[4][2];
     const double *wall_prof[4][2];
@@ -153,6 +152,7 @@ struct StepParams {
     int nbodies;
     int body_blocks[VPLBM_MAX_BODIES + 1];
     double body_radius[VPLBM_MAX_BODIES];
+    FixedConsts fx;               // the FP64 kernels' fixed-point constants (last: the others do not read them)
 };
 
 // Error bits latched in the control word.
