@@ -326,8 +326,11 @@ vplbm_status vplbm_get_body_k(vplbm_ctx *ctx, int k, double q[3], double v[3], l
  *                          refused); 0 x 0 keeps the current ones.  Its
  *                          populations equal the scalar kernel's bit for
  *                          bit; its force sums are added in another order.
- *                          Its first call allocates a workspace of a few MB
- *                          that the context keeps.
+ *                          The context keeps a workspace of a few MB for it,
+ *                          allocated when a state is set.  A launch takes
+ *                          every SM: contexts on different streams that
+ *                          should overlap choose another kernel (or are the
+ *                          members of a batch).
  * Nodes on the lattice edges and near the body always take the same code.
  * The results of different kernels agree to the rounding of the storage
  * precision. */

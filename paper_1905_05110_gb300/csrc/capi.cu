@@ -351,17 +351,28 @@ void setup_resident(vplbm_ctx *c)
     if (c->res_ok) c->res_bytes = resident_bytes(c->res_plan, c->precision, &c->res_poses, &c->res_parts);
 }
 
+// The resident kernel's workspace (a few MB, kept by the context).  Allocated
+// when a state is set, so that stepping allocates nothing.
+cudaError_t ensure_resident(vplbm_ctx *c)
+{
+    if (!c->res_ok || c->kernel != KERNEL_RESIDENT || c->res_ws) return cudaSuccess;
+    const cudaError_t e = cudaMalloc(&c->res_ws, c->res_bytes);
+    if (e != cudaSuccess) {
+        (void)cudaGetLastError();
+        c->res_ws = nullptr;
+        return e;
+    }
+    c->res_tag = 0;
+    return cudaSuccess;
+}
+
 // n <= RES_MAX_STEPS steps from the current one in one resident launch
 // (asynchronous); advances the step counter.
 cudaError_t launch_resident_steps(vplbm_ctx *c, int n)
 {
-    if (!c->res_ws) {
-        cudaError_t e = cudaMalloc(&c->res_ws, c->res_bytes);
-        if (e != cudaSuccess) {
-            c->res_ws = nullptr;
-            return e;
-        }
-        c->res_tag = 0;
+    {
+        const cudaError_t e = ensure_resident(c);   // a context stepped from the state at rest
+        if (e != cudaSuccess) return e;
     }
     if (c->res_tag == 0 || c->res_tag > 0xffffffffu - 2 * RES_MAX_STEPS) {   // new, or the tags are used up
         const cudaError_t e = cudaMemsetAsync(c->res_ws, 0, c->res_bytes, c->stream);
@@ -1004,6 +1015,7 @@ void *mapped_host(const void *host)
 vplbm_status vplbm_init_equilibrium(vplbm_ctx *c, const double *rho, const double *ux, const double *uy)
 {
     if (!c) return fail(VPLBM_EINVAL, "context is NULL");
+    (void)ensure_resident(c);   // without it the steps are launched one by one
     const size_t n = (size_t)c->nx * c->ny;
     double *tmp = nullptr;
     double *d[3] = {nullptr, nullptr, nullptr};
@@ -1030,6 +1042,7 @@ vplbm_status vplbm_init_equilibrium(vplbm_ctx *c, const double *rho, const doubl
 vplbm_status vplbm_set_populations(vplbm_ctx *c, const double *f)
 {
     if (!c || !f) return fail(VPLBM_EINVAL, "NULL argument");
+    (void)ensure_resident(c);
     try {
         std::vector<char> raw(c->pop_bytes, 0);
         full_to_stored(c, f, raw.data());
@@ -1468,6 +1481,7 @@ vplbm_status vplbm_load(vplbm_ctx *c, const char *path)
              fread(outlet.data(), sizeof(double), outlet.size(), fp) == outlet.size();
         fclose(fp);
         if (!ok) return fail(VPLBM_EIO, "%s is truncated", path);
+        (void)ensure_resident(c);
         const int par = (int)(h.nstep & 1);
         CUDA_TRY(cudaMemcpyAsync(const_cast<void *>(params_for(c, h.nstep).conv_in), outlet.data(),
                                  outlet.size() * sizeof(double), cudaMemcpyHostToDevice, c->stream));

@@ -50,7 +50,8 @@
 // Measured (GB300, us per step, one-step launches -> this kernel): FP32 256 x
 // 128 with a fixed disk 8.9 -> 2.4, 512 x 256 oscillating disk 8.7 -> 2.8, 512
 // x 256 disk on a spring (free) 14.1 -> 4.7, 700 x 400 9.0 -> 4.3, 1230 x 410
-// 10.5 -> 6.2; FP64 256 x 128 13.6 -> 8.1.  What is left: the update itself at
+// 10.5 -> 6.2; FP64 256 x 128 13.6 -> 6.6 (8.1 with the solid-node sums in FP64
+// instructions).  What is left: the update itself at
 // 7 nodes a thread (issue slots about half busy), and below 2 nodes a thread
 // the exchange and the three block barriers of a step.
 #define VPLBM_PLAIN_LOADS 1
@@ -454,6 +455,33 @@ __device__ __noinline__ void resident_tail(const ResidentLaunch &L, BodyState *s
 
 // ---- the tiles ---------------------------------------------------------
 
+// An exact sum of 64-bit fixed-point terms (FP64 storage, MRT: the solid-node
+// sums of a tile, since an FP64 addition costs a warp 65 clocks): the terms'
+// high words and their low words, summed apart.
+struct FxSum {
+    long long hi, lo;
+};
+__device__ __forceinline__ void acc_zero(FxSum &a) { a.hi = a.lo = 0; }
+__device__ __forceinline__ void acc_add(FxSum &a, FxSum b)
+{
+    a.hi += b.hi;
+    a.lo += b.lo;
+}
+__device__ __forceinline__ FxSum acc_shfl_down(FxSum a, int off)
+{
+    return {__shfl_down_sync(0xffffffffu, a.hi, off), __shfl_down_sync(0xffffffffu, a.lo, off)};
+}
+__device__ __forceinline__ FxSum fx_term(long long x) { return {x >> 32, (long long)(uint32_t)(uint64_t)x}; }
+// x y, y an int of up to 12 bits.
+__device__ __forceinline__ FxSum fx_term(long long x, int y) { return {(x >> 32) * y, (long long)(uint32_t)(uint64_t)x * y}; }
+// The sum in units of 2^k, as a double.
+__device__ __forceinline__ double fx_value(FxSum a, int k)
+{
+    const long long hi = a.hi + (a.lo >> 32);
+    if (hi + (1LL << 30) >= 0 && hi < 1LL << 30) return fx_signed_to((long long)((uint64_t)hi << 32) + (long long)(uint32_t)(uint64_t)a.lo, k);
+    return ((double)hi * 4294967296.0 + (double)(uint32_t)(uint64_t)a.lo) * ldexp(1.0, k);
+}
+
 // A node's word: its column (bits 0-11) and row (12-23) in the tile, and
 constexpr unsigned ND_VALID = 1u << 24, ND_LATTICE_EDGE = 1u << 25, ND_EDGE = 1u << 26, ND_CORNER = 1u << 27;
 __device__ __forceinline__ int nd_x(unsigned b) { return (int)(b & 0xfffu); }
@@ -529,6 +557,124 @@ __device__ __forceinline__ RingItem ring_item(int n, int m, int w, int h)
     return RingItem{south ? (m == 0 ? 2 : m == 1 ? 5 : 6) : (m == 0 ? 4 : m == 1 ? 7 : 8), south ? n : n - w, south ? -1 : h};
 }
 
+// FP64 storage, MRT: a tile's sums rows [q0, q0 + qn) of step k to their
+// readers.  Warp q - q0 reduces row q (a fixed order), then the first of them
+// sends the reaction (q0 = 0), the last four the forces to each of their
+// readers.  rows_mem: the rows, FxSum, or double where slow.  (A function of
+// its own; the FP32 kernels have theirs inlined, a call cost them 8 %.)
+template <typename Row>
+__device__ __forceinline__ Row reduce_row(const Row *row)
+{
+    const int lane = threadIdx.x & 31;
+    // four chains: an addition waits for the one before it in its chain only
+    Row c0 = row[lane], c1 = row[32 + lane], c2 = row[64 + lane], c3 = row[96 + lane];
+    for (int m = 4; m < RES_NT / 32; m += 4) {
+        acc_add(c0, row[m * 32 + lane]);
+        acc_add(c1, row[m * 32 + 32 + lane]);
+        acc_add(c2, row[m * 32 + 64 + lane]);
+        acc_add(c3, row[m * 32 + 96 + lane]);
+    }
+    acc_add(c0, c1);
+    acc_add(c2, c3);
+    acc_add(c0, c2);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) acc_add(c0, acc_shfl_down(c0, off));
+    return c0;
+}
+
+__device__ __noinline__ void publish_sums(const ResidentLaunch &L, const void *rows_mem, double *s_tot, int i0, int j0, int q0, int qn,
+                                          int k, int slot, int readers, bool slow, const BodyState *at)
+{
+    const int w0 = threadIdx.x >> 5, q = q0 + w0, lane = threadIdx.x & 31;
+    if (w0 >= qn) return;
+    if (!slow) {
+        const FxSum a = reduce_row(static_cast<const FxSum *>(rows_mem) + q * RES_NT);
+        if (lane == 0) s_tot[q] = q == 6 ? (double)a.lo : fx_value(a, L.p.fx.e - 59);
+    } else {
+        const double a = reduce_row(static_cast<const double *>(rows_mem) + q * RES_NT);
+        if (lane == 0) s_tot[q] = a;
+    }
+    __syncwarp();
+    asm volatile("bar.sync 1, %0;" ::"r"(32 * qn) : "memory");
+    const uint32_t tag = L.tag0 + (uint32_t)k;
+    const int m = lane & 3;
+    auto value = [&](int first) {   // sum first + m (the reaction has no fourth)
+        double a = first == 0 && m == 3 ? 0.0 : s_tot[first + m];
+        if (!slow && m == 2)        // the torque was taken about the tile's first node
+            a = fma(at->q[1] - (double)j0, s_tot[first], fma((double)i0 - at->q[0], s_tot[first + 1], a));
+        return make_uint2((uint32_t)__double2loint(a), (uint32_t)__double2hiint(a));
+    };
+    if (q0 == 0 && w0 == 0) {
+        const uint2 v = value(0);
+        if (lane < 4) send_pair(react_slot(L, k, slot) + 2 * m, v.x, v.y, tag);
+    }
+    if (q0 + qn == NPART - 1 && w0 >= qn - 4) {
+        const uint2 v = value(3);
+        // reader r by four lanes of warp (r >> 3) & 3 of four
+        for (int r = (w0 - (qn - 4)) * 8 + (lane >> 2); r < readers; r += 32)
+            send_pair(force_slot(L, k, slot, r) + 2 * m, v.x, v.y, tag);
+    }
+}
+
+// Whether a solid node's pulled and own populations are in the fixed-point
+// range, with a density and momentum that fx_update takes.
+__device__ __forceinline__ bool fx_in_range(const FixedConsts &k, const double f[NQ], const double *own)
+{
+    uint32_t top = 0, low = 0xffffffffu;
+    long long rho = 0, jx = 0, jy = 0;
+#pragma unroll
+    for (int a = 0; a < NQ; ++a) {
+        const uint64_t b = fx_bits(f[a]);
+        const uint32_t h = (uint32_t)(b >> 32), o = (uint32_t)(fx_bits(own[a]) >> 32);
+        top = max(top, max(h, o));
+        low = min(low, min(h, o));
+        const long long x = fx_from(b, k.e);
+        rho += x;
+        jx += cx_of(a) * x;
+        jy += cy_of(a) * x;
+    }
+    constexpr long long J = 201769274521386496LL;   // 0.35 2^59
+    return top < k.hi_max && low >= k.hi_min && rho >= 1LL << 58 && rho < 3LL << 58 && jx > -J && jx < J && jy > -J && jy < J;
+}
+
+// The update of a solid node in that range (out: its place in the stage), and
+// the reaction -rho a on a body of velocity bs->v that does not turn, in units
+// of 2^(E - 59).
+__device__ __noinline__ void fixed_solid_slow(const StepParams &p, const BodyState *bs, const double *f, double *c, long long &gx,
+                                              long long &gy)
+{
+    double out[NQ], kept[3];
+    mrt_native_f64(p, bs, true, 0.0, 0.0, f, out, kept);
+    for (int a = 0; a < NQ; ++a) c[a] = out[a];
+    const double s = ldexp(1.0, 59 - p.fx.e);   // |rho a| < 3: no overflow
+    gx = __double2ll_rn(-kept[0] * kept[1] * s);
+    gy = __double2ll_rn(-kept[0] * kept[2] * s);
+}
+__device__ __forceinline__ void fixed_solid(const StepParams &p, const BodyState *bs, const double f[NQ], double *c, long long &gx,
+                                            long long &gy)
+{
+    uint64_t bits[NQ];
+#pragma unroll
+    for (int a = 0; a < NQ; ++a) bits[a] = fx_bits(f[a]);
+    double out[NQ];
+    long long rho = 0, ax = 0, ay = 0;
+    if (fx_update<true>(p.fx, bits, true, fx_from_signed(fx_bits(bs->v[0])), fx_from_signed(fx_bits(bs->v[1])), out, rho, ax, ay)) {
+#pragma unroll
+        for (int a = 0; a < NQ; ++a) c[a] = out[a];
+        const long long r8 = (long long)((uint64_t)rho << 3);
+        gx = -fx_mul(r8, fx_split(2 * ax));
+        gy = -fx_mul(r8, fx_split(2 * ay));
+        return;
+    }
+    double in[NQ];
+#pragma unroll
+    for (int a = 0; a < NQ; ++a) in[a] = f[a];
+    fixed_solid_slow(p, bs, in, c, gx, gy);
+}
+
+template <bool FIXED, typename A> struct RowT { using R = A; };
+template <typename A> struct RowT<true, A> { using R = FxSum; };
+
 // One block per SM; K nodes of 9 (FP32) or 18 (FP64) registers wait for the
 // block between the pull and the update.
 template <int P, int COLL, int K>
@@ -544,7 +690,7 @@ __global__ void __launch_bounds__(RES_NT, 1) vp_mrt_resident(const __grid_consta
     extern __shared__ __align__(16) unsigned char res_smem[];
     __shared__ __align__(16) BodyState s_bs[RES_TAIL_WARPS + 1];   // tiles: [step parity]; the tail: one per warp, its counters
     __shared__ int s_abort[2];   // a ring wait, the pose wait gave up
-    __shared__ A s_force[4];     // a free body's forces and node count in this tile
+    __shared__ A s_tot[NPART - 1];   // the tile's sums
     const StepParams &p = L.p;
     const ResidentPlan &t = L.t;
     const int tid = threadIdx.x;
@@ -552,8 +698,13 @@ __global__ void __launch_bounds__(RES_NT, 1) vp_mrt_resident(const __grid_consta
         if (!L.mute) resident_tail<P>(L, s_bs);
         return;
     }
-    A (*rows)[NT] = reinterpret_cast<A (*)[NT]>(res_smem);   // [7 sums][thread]
-    S *stage = reinterpret_cast<S *>(res_smem + (NPART - 1) * NT * sizeof(A));
+    // solid-node sums: FP32 storage float-float, FP64 storage fixed point
+    // (FIXED) or, where a solid node is out of its range, FP64
+    constexpr bool FIXED = P == VPLBM_F64 && COLL == VPLBM_COLLISION_MRT;
+    using R = typename RowT<FIXED, A>::R;
+    R (*rows)[NT] = reinterpret_cast<R (*)[NT]>(res_smem);   // [7 sums][thread]
+    A (*slow_rows)[NT] = reinterpret_cast<A (*)[NT]>(res_smem);
+    S *stage = reinterpret_cast<S *>(res_smem + (NPART - 1) * NT * (P == VPLBM_F64 ? 16 : 8));
     const int pitch = (t.mw + 2) | 1;   // odd: a column of nodes is spread over the banks
     T *outlet = reinterpret_cast<T *>(stage + (size_t)pitch * (t.mh + 2) * NQ);   // [3][mh]
     // per edge node of the tile (in the order of the threads that own them):
@@ -670,49 +821,55 @@ __global__ void __launch_bounds__(RES_NT, 1) vp_mrt_resident(const __grid_consta
     // the sums rows [q0, q0 + qn) of step k to their readers: warp q reduces
     // row q (NT / 32 adds per lane in thread order, then a shuffle tree), and
     // for a free body's forces one warp sends them all
-    auto publish = [&](int q0, int qn, int k, int slot, int readers) {
-        const int q = q0 + (tid >> 5), lane = tid & 31;
-        if (q >= q0 + qn) return;
-        A a;
-        {   // four chains: an addition waits for the one before it in its chain only
-            A c[4];
+    auto publish = [&](int q0, int qn, int k, int slot, int readers, bool slow, const BodyState *at) {
+        if constexpr (FIXED) {
+            publish_sums(L, res_smem, s_tot, i0, j0, q0, qn, k, slot, readers, slow, at);
+            return;
+        } else {
+            const int q = q0 + (tid >> 5), lane = tid & 31;
+            if (q >= q0 + qn) return;
+            A a;
+            {   // four chains: an addition waits for the one before it in its chain only
+                A c[4];
 #pragma unroll
-            for (int m = 0; m < 4; ++m) c[m] = rows[q][m * 32 + lane];
-            for (int m = 4; m < NT / 32; m += 4)
+                for (int m = 0; m < 4; ++m) c[m] = rows[q][m * 32 + lane];
+                for (int m = 4; m < NT / 32; m += 4)
 #pragma unroll
-                for (int e = 0; e < 4; ++e) acc_add(c[e], rows[q][(m + e) * 32 + lane]);
-            acc_add(c[0], c[1]);
-            acc_add(c[2], c[3]);
-            acc_add(c[0], c[2]);
-            a = c[0];
-        }
+                    for (int e = 0; e < 4; ++e) acc_add(c[e], rows[q][(m + e) * 32 + lane]);
+                acc_add(c[0], c[1]);
+                acc_add(c[2], c[3]);
+                acc_add(c[0], c[2]);
+                a = c[0];
+            }
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) acc_add(a, acc_shfl_down(a, off));
-        const uint32_t tag = L.tag0 + (uint32_t)k;
-        if (readers > 1) {   // forces, warps 0 .. 3
-            if (lane == 0) s_force[q - 3] = a;
-            __syncwarp();
-            asm volatile("bar.sync 1, 128;" ::: "memory");
-            const uint2 v = reinterpret_cast<const uint2 *>(s_force)[lane & 3];
-            // reader r by four lanes of warp (r >> 3) & 3
-            for (int r = (tid >> 5) * 8 + (lane >> 2); r < readers; r += 32)
-                send_pair(force_slot(L, k, slot, r) + 2 * (lane & 3), v.x, v.y, tag);
-        } else if (lane == 0) {
-            uint32_t v[2];
-            memcpy(v, &a, 8);
-            send_pair(q < 3 ? react_slot(L, k, slot) + 2 * q : force_slot(L, k, slot, 0) + 2 * (q - 3), v[0], v[1], tag);
-            if (q == 2) send_pair(react_slot(L, k, slot) + 6, 0u, 0u, tag);   // the fourth of four
+            for (int off = 16; off > 0; off >>= 1) acc_add(a, acc_shfl_down(a, off));
+            const uint32_t tag = L.tag0 + (uint32_t)k;
+            if (readers > 1) {   // forces, warps 0 .. 3
+                if (lane == 0) s_tot[q - 3] = a;
+                __syncwarp();
+                asm volatile("bar.sync 1, 128;" ::: "memory");
+                const uint2 v = reinterpret_cast<const uint2 *>(s_tot)[lane & 3];
+                // reader r by four lanes of warp (r >> 3) & 3
+                for (int r = (tid >> 5) * 8 + (lane >> 2); r < readers; r += 32)
+                    send_pair(force_slot(L, k, slot, r) + 2 * (lane & 3), v.x, v.y, tag);
+            } else if (lane == 0) {
+                uint32_t v[2];
+                memcpy(v, &a, 8);
+                send_pair(q < 3 ? react_slot(L, k, slot) + 2 * q : force_slot(L, k, slot, 0) + 2 * (q - 3), v[0], v[1], tag);
+                if (q == 2) send_pair(react_slot(L, k, slot) + 6, 0u, 0u, tag);   // the fourth of four
+            }
         }
     };
     int owed = -1;              // the slot whose sums of the last step are still to be published
     Pair ahead{0, 0};           // words of the next pose, read early (published already on a prescribed path)
     bool own_pose = false;      // this step's pose was computed here
+    bool slow = false;          // FIXED: a solid node of the tile is out of range
 
     for (int k = 0; k < L.nsteps; ++k) {
         const uint32_t tag = L.tag0 + (uint32_t)k;
         BodyState *bs = s_bs + (k & 1);
         __syncthreads();   // step k - 1 is in the stage
-        if (owed >= 0) publish(0, early ? 3 : NPART - 1, k - 1, owed, 1);
+        if (owed >= 0) publish(0, early ? 3 : NPART - 1, k - 1, owed, 1, slow, s_bs + ((k - 1) & 1));
         // ---- pull of the inner nodes, which need no neighbour ----
         T f[K][NQ];
         auto pull_inner = [&](unsigned b, T g[NQ]) {
@@ -850,45 +1007,6 @@ __global__ void __launch_bounds__(RES_NT, 1) vp_mrt_resident(const __grid_consta
         const int slot = (ty - rect.y) * rect.z + tx - rect.x;
         if (sums && !near && tid < 8)   // no solid node anywhere
             send_pair((tid < 4 ? force_slot(L, k, 0, 0) : react_slot(L, k, 0)) + 2 * (tid & 3), 0u, 0u, tag);
-        unsigned solid = 0;   // my solid nodes
-        if (near) {
-            // the momentum exchanged: pulled minus own, before the own
-            // populations are overwritten
-            A ex_[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) acc_zero(ex_[q]);
-#pragma unroll
-            for (int it = 0; it < K; ++it) {
-                const unsigned b = node[it];
-                const int i = i0 + nd_x(b), j = j0 + nd_y(b);
-                if (!(b & ND_VALID) || i < range.x || i > range.y || j < range.z || j > range.w) continue;
-                T dxl = 0, dyl = 0;
-                if (!body_chi<P, SHAPE_ANY>(p.body, p.r2f, bs, i, j, dxl, dyl)) continue;
-                solid |= 1u << it;
-                const S *c = stage + nd_off(b, pitch);
-                V ex = 0, ey = 0;
-#pragma unroll
-                for (int a = 1; a < NQ; ++a) {
-                    const V g = (V)f[it][a] - (V)c[a];
-                    ex += cx_of(a) * g;
-                    ey += cy_of(a) * g;
-                }
-                acc_add(ex_[0], ex);
-                acc_add(ex_[1], ey);
-                acc_add(ex_[2], (V)dxl * ey - (V)dyl * ex);
-                acc_add(ex_[3], (V)1);
-            }
-#pragma unroll
-            for (int q = 0; q < 4; ++q) rows[3 + q][tid] = ex_[q];
-            if (early) {
-                __syncthreads();
-                publish(3, 4, k, slot, 1 + rect.z * rect.w);
-            }
-        }
-        // the penalization's reaction, summed over my solid nodes
-        A part[3];
-#pragma unroll
-        for (int q = 0; q < 3; ++q) acc_zero(part[q]);
         auto lever = [&](unsigned b, T &dx, T &dy) {
             if constexpr (P == VPLBM_F64) {
                 dx = (double)(i0 + nd_x(b)) - bs->q[0];
@@ -898,12 +1016,103 @@ __global__ void __launch_bounds__(RES_NT, 1) vp_mrt_resident(const __grid_consta
                 dy = (float)(j0 + nd_y(b) - bs->yi) - bs->yf;
             }
         };
+        unsigned solid = 0;   // my solid nodes
+        if (near) {
+            // the momentum exchanged by a solid node: pulled minus own, before
+            // the own populations are overwritten
+            A ex_[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc_zero(ex_[q]);
+            auto exchange = [&](unsigned b, const T g[NQ], T dx, T dy) {
+                const S *c = stage + nd_off(b, pitch);
+                V ex = 0, ey = 0;
+#pragma unroll
+                for (int a = 1; a < NQ; ++a) {
+                    const V d = (V)g[a] - (V)c[a];
+                    ex += cx_of(a) * d;
+                    ey += cy_of(a) * d;
+                }
+                acc_add(ex_[0], ex);
+                acc_add(ex_[1], ey);
+                acc_add(ex_[2], (V)dx * ey - (V)dy * ex);
+                acc_add(ex_[3], (V)1);
+            };
+            bool bad = false;
+#pragma unroll
+            for (int it = 0; it < K; ++it) {
+                const unsigned b = node[it];
+                const int i = i0 + nd_x(b), j = j0 + nd_y(b);
+                if (!(b & ND_VALID) || i < range.x || i > range.y || j < range.z || j > range.w) continue;
+                T dxl = 0, dyl = 0;
+                if (!body_chi<P, SHAPE_ANY>(p.body, p.r2f, bs, i, j, dxl, dyl)) continue;
+                solid |= 1u << it;
+                if constexpr (FIXED) bad = bad || !fx_in_range(p.fx, f[it], stage + nd_off(b, pitch));
+                else exchange(b, f[it], dxl, dyl);
+            }
+            if constexpr (FIXED) {
+                // a body that turns, or moves fast, takes the FP64 code too
+                const uint64_t v0 = fx_bits(bs->v[0]), v1 = fx_bits(bs->v[1]);
+                bad = bad || !p.fx.ok || p.fx.forced || bs->v[2] != 0.0 || ((v0 >> 32) & 0x7fffffffu) >= 0x3fd00000u ||
+                      ((v1 >> 32) & 0x7fffffffu) >= 0x3fd00000u;
+                slow = __syncthreads_or(bad);
+            }
+            if constexpr (FIXED) {
+                if (!slow) {
+                    FxSum sum[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) acc_zero(sum[q]);
+#pragma unroll
+                    for (int it = 0; it < K; ++it) {
+                        if (!((solid >> it) & 1u)) continue;
+                        const unsigned b = node[it];
+                        const S *c = stage + nd_off(b, pitch);
+                        long long ex = 0, ey = 0;
+#pragma unroll
+                        for (int a = 1; a < NQ; ++a) {
+                            const long long g = fx_from(fx_bits(f[it][a]), p.fx.e) - fx_from(fx_bits(c[a]), p.fx.e);
+                            if (cx_of(a)) ex += cx_of(a) > 0 ? g : -g;
+                            if (cy_of(a)) ey += cy_of(a) > 0 ? g : -g;
+                        }
+                        acc_add(sum[0], fx_term(ex));
+                        acc_add(sum[1], fx_term(ey));
+                        acc_add(sum[2], fx_term(ey, nd_x(b)));
+                        acc_add(sum[2], fx_term(ex, -nd_y(b)));
+                        sum[3].lo += 1;
+                    }
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) rows[3 + q][tid] = sum[q];
+                } else {
+#pragma unroll
+                    for (int it = 0; it < K; ++it) {
+                        if (!((solid >> it) & 1u)) continue;
+                        T dx, dy;
+                        lever(node[it], dx, dy);
+                        exchange(node[it], f[it], dx, dy);
+                    }
+                }
+            }
+            if (!FIXED || slow) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) slow_rows[3 + q][tid] = ex_[q];
+            }
+            if (early) {
+                __syncthreads();
+                publish(3, 4, k, slot, 1 + rect.z * rect.w, slow, bs);
+            }
+        }
+        // the penalization's reaction, summed over my solid nodes
+        A part[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) acc_zero(part[q]);
         auto react = [&](T dx, T dy, T rho, T ax, T ay) {
             const V fx = -(V)rho * (V)ax, fy = -(V)rho * (V)ay;
             acc_add(part[0], fx);
             acc_add(part[1], fy);
             acc_add(part[2], (V)dx * fy - (V)dy * fx);
         };
+        FxSum fpart[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) acc_zero(fpart[q]);
         constexpr bool PAIRS = P == VPLBM_F32_DEV && COLL == VPLBM_COLLISION_MRT;
         if constexpr (PAIRS) {
             // two of my nodes at a time on paired lanes
@@ -940,19 +1149,38 @@ __global__ void __launch_bounds__(RES_NT, 1) vp_mrt_resident(const __grid_consta
 #pragma unroll
         for (int it = PAIRS ? K / 2 * 2 : 0; it < K; ++it) {
             const unsigned b = node[it];
-            if (b & ND_VALID) {
+            auto update_one = [&]() {
                 S *c = stage + nd_off(b, pitch);
                 T dxl = 0, dyl = 0, cr = 0, cax = 0, cay = 0;
                 const bool chi = (solid >> it) & 1u;
+                if constexpr (FIXED) {
+                    if (chi && !slow) {
+                        long long gx = 0, gy = 0;
+                        fixed_solid(p, bs, f[it], c, gx, gy);   // -rho a
+                        acc_add(fpart[0], fx_term(gx));
+                        acc_add(fpart[1], fx_term(gy));
+                        acc_add(fpart[2], fx_term(gy, nd_x(b)));
+                        acc_add(fpart[2], fx_term(gx, -nd_y(b)));
+                        return;
+                    }
+                }
                 if (chi) lever(b, dxl, dyl);
                 node_collide_to<P, COLL>(p, bs, chi, dxl, dyl, f[it], [&](int a, T v) { c[a] = v; }, cr, cax, cay);
                 if (chi) react(dxl, dyl, cr, cax, cay);
-            }
+            };
+            if (b & ND_VALID) update_one();
             if (it == 0) post_edge();
         }
         if (near) {
 #pragma unroll
-            for (int q = 0; q < 3; ++q) rows[q][tid] = part[q];
+            for (int q = 0; q < 3; ++q) {
+                if constexpr (FIXED) {
+                    if (!slow) rows[q][tid] = fpart[q];
+                    else slow_rows[q][tid] = part[q];
+                } else {
+                    rows[q][tid] = part[q];
+                }
+            }
         }
         owed = near ? slot : -1;
         own_pose = early && near && send;
@@ -960,7 +1188,7 @@ __global__ void __launch_bounds__(RES_NT, 1) vp_mrt_resident(const __grid_consta
     }
     if (owed >= 0) {
         __syncthreads();
-        publish(0, early ? 3 : NPART - 1, L.nsteps - 1, owed, 1);
+        publish(0, early ? 3 : NPART - 1, L.nsteps - 1, owed, 1, slow, s_bs + ((L.nsteps - 1) & 1));
     }
 
     // the state after the last step (every thread its own nodes)
@@ -1025,7 +1253,7 @@ int resident_k(int precision, int w, int h, int *edge_at, int *smem)
     for (int k = 1; k <= maxk; ++k) {
         if ((long long)w * h > (long long)k * RES_NT) continue;
         // the sums' rows, the stage, the outlet record; then the edge tables
-        const long long at = ((NPART - 1) * (long long)RES_NT * 8 + (NQ * ((w + 2LL) | 1) * (h + 2LL) + 3LL * h) * es + 15) / 16 * 16;
+        const long long at = ((NPART - 1) * (long long)RES_NT * 2 * es + (NQ * ((w + 2LL) | 1) * (h + 2LL) + 3LL * h) * es + 15) / 16 * 16;
         const long long bytes = at + 2LL * (w + h) * (NQ * 2 * es + 7 * 4);
         if (bytes > 225 * 1024 || (precision == VPLBM_F64 ? 8 : 4) * (w + h) > RES_RECV * RES_NT || 2 * (w + h) > RES_NT || w < 3 ||
             h < 3 || w > 4095 || h > 4095)
