@@ -558,9 +558,7 @@ def run_other_workload(name, steps, torch, stream):
     t = time_device(sim, steps, stream, torch)
     sim.sync()
     half = steps // 2
-    # (a small lattice: its resident launches, up to 4096 steps each, count as one_step)
-    out = {"workload": p["name"], "mlups": nodes * steps / t / 1e6, "steps": steps, "launch": list(launch),
-           "kernel_launches": sim.kernel_launches()}
+    out = {"workload": p["name"], "mlups": nodes * steps / t / 1e6, "steps": steps, "launch": list(launch)}
     bodies = p.get("bodies") or [p["body"]]
     per_body = []
     for k, b in enumerate(bodies):

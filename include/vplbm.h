@@ -318,8 +318,8 @@ vplbm_status vplbm_get_body_k(vplbm_ctx *ctx, int k, double q[3], double v[3], l
  *                          what a context of such a lattice does by default
  *                          and what vplbm_autotune may choose (vplbm_get_launch
  *                          then names the kernel of its single launches).  One cooperative
- *                          launch runs up to 4096 steps; it counts as one
- *                          VPLBM_LAUNCH_ONE_STEP launch.  (block_x,
+ *                          launch runs up to 4096 steps; the launch counts
+ *                          count its steps, one VPLBM_LAUNCH_ONE_STEP each.  (block_x,
  *                          block_y): the blocks of steps that have to be
  *                          launched one by one (on a stream that is being
  *                          captured, or where a cooperative launch is
@@ -360,7 +360,8 @@ vplbm_status vplbm_autotune(vplbm_ctx *ctx, int steps_per_trial);
  * VPLBM_EUNSUPPORTED unless one of the two is selected. */
 vplbm_status vplbm_inject_wait_timeout(vplbm_ctx *ctx, int enable);
 
-/* Number of step-kernel launches made by vplbm_step since creation
+/* Number of step-kernel launches made by vplbm_step since creation (a
+ * resident launch counts once for each of its steps)
  * (vplbm_load restores the count saved in the checkpoint). */
 vplbm_status vplbm_get_launch_count(vplbm_ctx *ctx, long long *launches);
 
@@ -368,8 +369,8 @@ vplbm_status vplbm_get_launch_count(vplbm_ctx *ctx, long long *launches);
  * vplbm_get_kernel_launches):
  *  VPLBM_LAUNCH_ONE_STEP   one time step on a scalar step kernel (any
  *                          register budget, shape, or several bodies) or
- *                          on the node-pair kernel; or one launch of the
- *                          resident kernel (its steps together);
+ *                          on the node-pair kernel, or one time step of a
+ *                          resident launch;
  *  VPLBM_LAUNCH_TWO_STEP   two time steps on the two-step kernel;
  *  VPLBM_LAUNCH_LOOKAHEAD  the one-thread launch that computes pose n + 1
  *                          of a prescribed path ahead of a run of two-step

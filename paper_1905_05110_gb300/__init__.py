@@ -669,7 +669,7 @@ class Simulation:
 
     @property
     def launches(self) -> int:
-        """Kernel launches made by step() since creation."""
+        """Kernel launches made by step() since creation (a resident launch counts once per step)."""
         return vplbm_get_launch_count(self.ctx)
 
     def kernel_launches(self) -> dict:

@@ -827,8 +827,9 @@ vplbm_status step_impl(vplbm_ctx *c, long long n)
                 ctx_disable_resident(c);
                 break;
             }
-            c->kcount[VPLBM_LAUNCH_ONE_STEP] += 1;
-            c->launches += 1;
+            // counted by steps, as the launches they stand for
+            c->kcount[VPLBM_LAUNCH_ONE_STEP] += m;
+            c->launches += m;
             n -= m;
         }
     }
