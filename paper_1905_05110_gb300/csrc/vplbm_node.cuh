@@ -92,11 +92,6 @@ template <typename T> __device__ __forceinline__ T par(double d, float f);
 template <> __device__ __forceinline__ double par<double>(double d, float) { return d; }
 template <> __device__ __forceinline__ float par<float>(double, float f) { return f; }
 
-// Host-folded relaxation factors in the arithmetic type of the kernel.
-template <typename T> __device__ __forceinline__ const auto &folded(const StepParams &p);
-template <> __device__ __forceinline__ const auto &folded<float>(const StepParams &p) { return p.pc; }
-template <> __device__ __forceinline__ const auto &folded<double>(const StepParams &p) { return p.pcd; }
-
 __device__ __forceinline__ double wall_u(const StepParams &p, int side, int comp, int k)
 {
     const double *prof = p.wall_prof[side][comp];
@@ -822,7 +817,7 @@ __device__ __forceinline__ bool node_collide_to(const StepParams &p, const BodyS
         cay = kept[2];
         return chi;
     }
-    // sums shared by the moments (rows of Eq. 15)
+    // BGK: sums shared by the moments (rows of Eq. 15)
     const T d13 = f[1] - f[3], d24 = f[2] - f[4], b13 = f[1] + f[3], b24 = f[2] + f[4];
     const T d56 = f[5] - f[6], d87 = f[8] - f[7], a56 = f[5] + f[6], a78 = f[7] + f[8];
     const T sx = d56 + d87, ty = a56 - a78, sa = b13 + b24, sd = a56 + a78;
