@@ -46,31 +46,37 @@
 namespace vplbm {
 namespace {
 
-// A factor r in (-1/2, 1/2) as r = hi 2^-32 + lo 2^-64 with signed digits.
+// A factor r as r = hi 2^-32 + lo 2^-64 with signed digits, which hold
+// -1/2 <= r < 1/2 - 2^-33.
 struct FxFactor {
     int hi, lo;
 };
 
 // Host-folded constants of the fixed-point update (uniform over a run).
 struct FixedConsts {
-    int ok;                     // the run's rho0 and g are in range
+    int ok;                     // the run's rho0, g and factors are in range
     int e;                      // E
     double unit;                // 2^(E - 59)
     unsigned hi_min, hi_max;    // high words of the doubles in [2^(E-32), 2^E)
     FxFactor r1, r2, r4, r6, r7, r8;   // s1/36, s2/12, s4/12, s6/12, s7/4, s8/4
     // forcing: (1 - s/2) / 6 for e and eps, / 12 for q, / 2 and / 4 for the
-    // stress, 1/6, and pen_k / 4
-    FxFactor h1, h2, h4, h6, h7, h8, sixth, k4;
+    // stress, 1/6, and pen_k / 8 (pen_k = 1 / (eta + 1/2) tends to 2)
+    FxFactor h1, h2, h4, h6, h7, h8, sixth, k8;
     long long gvx, gvy;         // g 2^60
     int forced;                 // g is not zero
     long long rho0;             // in units of 2^(E - 59)
     FxFactor w0, w1, w2;        // the weights
 };
 
-inline FxFactor fx_factor(double r)
+// ok is cleared where the digits do not hold r.
+inline FxFactor fx_factor(double r, int &ok)
 {
+    FxFactor f = {0, 0};
+    if (!(fabs(r) <= 0.5 - 0x1p-32)) {
+        ok = 0;
+        return f;
+    }
     const long long v = llrint(ldexp(r, 64));
-    FxFactor f;
     f.lo = (int)(uint32_t)(uint64_t)v;
     f.hi = (int)((v - (long long)f.lo) >> 32);
     return f;
@@ -83,23 +89,26 @@ inline void fold_fixed(FixedConsts &k, const double *s, double rho0, double gx, 
     const double m = frexp(rho0, &e);   // rho0 = m 2^e, m in [1/2, 1)
     if (m == 0.5) e -= 1;               // rho0 in (2^(E-1), 2^E]
     if (!(rho0 > 0.0) || e < -400 || e > 400 || !(fabs(gx) < 0.0625) || !(fabs(gy) < 0.0625)) return;
-    k.ok = 1;
     k.e = e;
     k.unit = ldexp(1.0, e - 59);
     k.hi_min = (unsigned)(991 + e) << 20;
     k.hi_max = (unsigned)(1023 + e) << 20;
-    k.r1 = fx_factor(s[1] / 36.0); k.r2 = fx_factor(s[2] / 12.0); k.r4 = fx_factor(s[4] / 12.0);
-    k.r6 = fx_factor(s[6] / 12.0); k.r7 = fx_factor(s[7] / 4.0); k.r8 = fx_factor(s[8] / 4.0);
-    k.h1 = fx_factor((1.0 - 0.5 * s[1]) / 6.0); k.h2 = fx_factor((1.0 - 0.5 * s[2]) / 6.0);
-    k.h4 = fx_factor((1.0 - 0.5 * s[4]) / 12.0); k.h6 = fx_factor((1.0 - 0.5 * s[6]) / 12.0);
-    k.h7 = fx_factor((1.0 - 0.5 * s[7]) / 2.0); k.h8 = fx_factor((1.0 - 0.5 * s[8]) / 4.0);
-    k.sixth = fx_factor(1.0 / 6.0);
-    k.k4 = fx_factor(0.25 * pen_k);     // pen_k = 1 / (eta + 1/2) < 2
+    // a rate s_7 or s_8 within 2^-30 of 2, or an s_7 below 2^-30, makes a
+    // factor that does not fit; such a run takes the FP64 instructions
+    int ok = 1;
+    k.r1 = fx_factor(s[1] / 36.0, ok); k.r2 = fx_factor(s[2] / 12.0, ok); k.r4 = fx_factor(s[4] / 12.0, ok);
+    k.r6 = fx_factor(s[6] / 12.0, ok); k.r7 = fx_factor(s[7] / 4.0, ok); k.r8 = fx_factor(s[8] / 4.0, ok);
+    k.h1 = fx_factor((1.0 - 0.5 * s[1]) / 6.0, ok); k.h2 = fx_factor((1.0 - 0.5 * s[2]) / 6.0, ok);
+    k.h4 = fx_factor((1.0 - 0.5 * s[4]) / 12.0, ok); k.h6 = fx_factor((1.0 - 0.5 * s[6]) / 12.0, ok);
+    k.h7 = fx_factor((1.0 - 0.5 * s[7]) / 2.0, ok); k.h8 = fx_factor((1.0 - 0.5 * s[8]) / 4.0, ok);
+    k.sixth = fx_factor(1.0 / 6.0, ok);
+    k.k8 = fx_factor(0.125 * pen_k, ok);
     k.gvx = llrint(ldexp(gx, 60));
     k.gvy = llrint(ldexp(gy, 60));
     k.forced = gx != 0.0 || gy != 0.0;
     k.rho0 = llrint(ldexp(rho0, 59 - e));
-    k.w0 = fx_factor(4.0 / 9.0); k.w1 = fx_factor(1.0 / 9.0); k.w2 = fx_factor(1.0 / 36.0);
+    k.w0 = fx_factor(4.0 / 9.0, ok); k.w1 = fx_factor(1.0 / 9.0, ok); k.w2 = fx_factor(1.0 / 36.0, ok);
+    k.ok = ok;
 }
 
 VPLBM_FX int fx_clz(uint32_t x)
@@ -249,8 +258,8 @@ VPLBM_FX bool fx_forced_here(const FixedConsts &k, bool chi, FxForced &w)
         const long long lx = w.usx - wx, ly = w.usy - wy;
         constexpr long long Q = 1LL << 59;
         if ((uint64_t)(lx + Q) >= (uint64_t)(2 * Q) || (uint64_t)(ly + Q) >= (uint64_t)(2 * Q)) return false;
-        ax = fx_mul(2 * lx, k.k4);
-        ay = fx_mul(2 * ly, k.k4);
+        ax = fx_mul(4 * lx, k.k8);   // |4 l| < 2^61
+        ay = fx_mul(4 * ly, k.k8);
     }
     const FxFactor ux = fx_split(wx + ax), uy = fx_split(wy + ay);   // u = v + a / 2
     const long long r8 = (long long)((uint64_t)w.rho << 3);

@@ -1,0 +1,132 @@
+"""The fixed-point arithmetic of FP64 storage (csrc/fixed64.cuh), compiled for
+the host, against the method's equations in extended precision.
+
+Tolerance of an update: FP64 instructions make a chain of about ten roundings
+of terms of at most 4 rho (the e and eps rows of Eq. 15), below 10 * 2^-53 *
+4 rho = 4.4e-15 rho, and the fixed-point update is to be no worse.
+"""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1905_05110_gb300", "csrc")
+UPDATE_TOL = 4.4e-15
+
+SHIM = r"""
+#include "fixed64.cuh"
+using namespace vplbm;
+
+// n nodes f[9]: the update into out (a node that is out of range: done = 0)
+extern "C" int fx_host_update(const double *s, double rho0, double gx, double gy, double pen_k, long n, int chi,
+                              const double *f, const double *us, double *out, double *acc, int *done)
+{
+    FixedConsts k;
+    fold_fixed(k, s, rho0, gx, gy, pen_k);
+    for (long m = 0; m < n; ++m) {
+        uint64_t b[9];
+        for (int a = 0; a < 9; ++a) b[a] = fx_bits(f[9 * m + a]);
+        long long rho = 0, ax = 0, ay = 0;
+        done[m] = k.ok && fx_update(k, b, chi != 0, llrint(ldexp(us[2 * m], 61)), llrint(ldexp(us[2 * m + 1], 61)), out + 9 * m,
+                                    rho, ax, ay);
+        acc[2 * m] = ldexp((double)ax, -60);
+        acc[2 * m + 1] = ldexp((double)ay, -60);
+    }
+    return k.ok;
+}
+"""
+
+M = np.array([[1, 1, 1, 1, 1, 1, 1, 1, 1], [-4, -1, -1, -1, -1, 2, 2, 2, 2], [4, -2, -2, -2, -2, 1, 1, 1, 1],
+              [0, 1, 0, -1, 0, 1, -1, -1, 1], [0, -2, 0, 2, 0, 1, -1, -1, 1], [0, 0, 1, 0, -1, 1, 1, -1, -1],
+              [0, 0, -2, 0, 2, 1, 1, -1, -1], [0, 1, -1, 1, -1, 0, 0, 0, 0], [0, 0, 0, 0, 0, 1, -1, 1, -1]])
+C = np.array([[0, 1, 0, -1, 0, 1, -1, -1, 1], [0, 0, 1, 0, -1, 1, 1, -1, -1]])
+W = np.array([4 / 9] + [1 / 9] * 4 + [1 / 36] * 4)
+LD = np.longdouble
+
+
+@pytest.fixture(scope="module")
+def host(tmp_path_factory):
+    d = tmp_path_factory.mktemp("fixed64")
+    src, lib = d / "shim.cpp", d / "shim.so"
+    src.write_text(SHIM)
+    # arithmetic on the integers wraps, as it does on the device
+    subprocess.run(["g++", "-O1", "-std=c++17", "-fwrapv", "-ffp-contract=off", "-fPIC", "-shared", f"-I{CSRC}", "-o", str(lib),
+                    str(src)], check=True)
+    return ctypes.CDLL(str(lib))
+
+
+def _ptr(a):
+    return a.ctypes.data_as(ctypes.c_void_p)
+
+
+def _rates(tau=0.7, **other):
+    s = [1 / tau, 1.1, 1.25, 1 / tau, 1.8, 1 / tau, 1.8, 1 / tau, 1 / tau]
+    for k, v in other.items():
+        s[int(k[1:])] = v
+    return np.array(s)
+
+
+def _nodes(n, rho0, seed, amp=0.1):
+    rng = np.random.default_rng(seed)
+    u = rng.uniform(-amp, amp, (2, n))
+    rho = rho0 * (1 + 0.02 * rng.uniform(-1, 1, n))
+    cu = C.T @ u
+    f = W[:, None] * rho * (1 + 3 * cu + 4.5 * cu * cu - 1.5 * (u * u).sum(0)) * (1 + 1e-3 * rng.uniform(-1, 1, (9, n)))
+    return np.ascontiguousarray(f.T), np.ascontiguousarray(rng.uniform(-0.05, 0.05, (n, 2)))
+
+
+def _update(host, f, us, s, rho0=1.0, g=(0.0, 0.0), eta=None):
+    n = len(f)
+    out, acc, done = np.zeros((n, 9)), np.zeros((n, 2)), np.zeros(n, np.int32)
+    pen = 0.0 if eta is None else 1.0 / (eta + 0.5)
+    host.fx_host_update(_ptr(s), ctypes.c_double(rho0), ctypes.c_double(g[0]), ctypes.c_double(g[1]), ctypes.c_double(pen),
+                        ctypes.c_long(n), int(eta is not None), _ptr(f), _ptr(us), _ptr(out), _ptr(acc), _ptr(done))
+    return out, acc, done.astype(bool)
+
+
+def _exact(f, us, s, g=(0.0, 0.0), eta=None):
+    """Collision with forcing (Eqs. 14-17, 22) of each node in extended precision."""
+    f = f.T.astype(LD)
+    m = M.astype(LD) @ f
+    rho, j = m[0], m[[3, 5]]
+    g = np.array(g, LD)[:, None]
+    u = j / rho + g / 2
+    a = np.zeros_like(u)
+    if eta is not None:
+        a = (us.T.astype(LD) - u) / (LD(eta) + LD(0.5))
+        u = u + a / 2
+    G = rho * (g + a)
+    u2, uG = (u * u).sum(0), (u * G).sum(0)
+    eq = np.array([rho, -2 * rho + 3 * rho * u2, rho - 3 * rho * u2, m[3], -rho * u[0], m[5], -rho * u[1],
+                   rho * (u[0] ** 2 - u[1] ** 2), rho * u[0] * u[1]])
+    F = np.array([0 * rho, 6 * uG, -6 * uG, G[0], -G[0], G[1], -G[1], 2 * (u[0] * G[0] - u[1] * G[1]), u[0] * G[1] + u[1] * G[0]])
+    sk = s.astype(LD)[:, None].copy()
+    sk[[0, 3, 5]] = 0
+    d = sk * (eq - m) + (1 - sk / 2) * F
+    return (f + (M / (M * M).sum(1)[:, None].astype(LD)).T.astype(LD) @ d).T, a.T
+
+
+@pytest.mark.parametrize("eta", [1e-3, 1e-9, 1.2e-10, 1.1e-10, 1e-12, 1e-20])
+@pytest.mark.parametrize("rho0", [1.0, 0.7])
+def test_penalization_factor_of_every_eta(host, eta, rho0):
+    f, us = _nodes(500, rho0, 1)
+    out, acc, done = _update(host, f, us, _rates(), rho0, eta=eta)
+    assert done.all()   # in fixed point, at any eta
+    want, a = _exact(f, us, _rates(), eta=eta)
+    assert np.max(np.abs(acc - a)) < 1e-15
+    assert np.max(np.abs(out - want)) < UPDATE_TOL * 1.1 * rho0
+
+
+@pytest.mark.parametrize("rates", [{"s7": 2 - 1e-10}, {"s8": 2 - 1e-10}, {"s7": 1e-10}, {"s8": 1e-10}, {"s7": 2 - 1e-9},
+                                   {"s7": 1e-9}, {"s1": 2 - 1e-15, "s4": 1e-15}])
+@pytest.mark.parametrize("g", [(0.0, 0.0), (1e-3, -2e-3)])
+@pytest.mark.parametrize("eta", [None, 1e-3])
+def test_rates_at_the_ends_of_their_range(host, rates, g, eta):
+    """Rates in (0, 2) up to its ends: the right update, or left to the FP64 instructions."""
+    f, us = _nodes(500, 1.0, 2)
+    s = _rates(**rates)
+    out, _, done = _update(host, f, us, s, g=g, eta=eta)
+    want, _ = _exact(f, us, s, g=g, eta=eta)
+    assert np.max(np.abs(out - want)[done], initial=0.0) < UPDATE_TOL * 1.1

@@ -1,0 +1,80 @@
+"""FP64 storage at the ends of the accepted penalization and relaxation
+parameters, on every stepping path, against the oracle.
+
+One step; tolerance 5.3e-14 of the largest population (two chains of ten
+roundings of terms of at most 4 rho, the populations of rho <= 2 rho0 above
+rho0 / 3).
+"""
+import numpy as np
+import pytest
+
+import workloads as wl
+from helpers import make_pair, moving_bodies, rel_err
+
+pytestmark = pytest.mark.gpu
+
+TOL = 5.3e-14
+ENDS = [dict(eta=e) for e in (1e-9, 1.2e-10, 1.1e-10, 1e-12, 1e-20)] + [
+    {"s7": 2 - 1e-10}, {"s8": 2 - 1e-10}, {"s7": 1e-10, "g": (1e-3, 0.0)}, {"s8": 1e-10, "g": (1e-3, 0.0)}]
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _library(gpu_library):
+    return gpu_library
+
+
+def _ended(p, end):
+    p["s"] = list(p["s"])
+    for k, v in end.items():
+        if k == "eta":
+            p["eta"] = v
+        elif k == "g":
+            p["g_fluid"] = v
+        else:
+            p["s"][int(k[1:])] = v
+    return p
+
+
+@pytest.mark.parametrize("end", ENDS, ids=str)
+@pytest.mark.parametrize("path", ["scalar", "resident", "several"])
+def test_one_step_at_the_ends_of_the_parameters(end, path):
+    nx, ny = 67, 45
+    bodies = moving_bodies(nx, ny)
+    p = _ended(wl.mixed_bc_box(nx, ny, seed=3, body=dict(bodies["free"], omega=0.0), tau=0.7), end)
+    if path == "several":
+        p["bodies"] = [dict(p.pop("body"), radius=6.0), dict(bodies["imposed"], radius=5.0, x=50.0, y=30.0)]
+    gpu, orc = make_pair(p, "f64", f0=wl.random_populations(nx, ny, seed=5, amp=0.03))
+    if path != "several":
+        gpu.set_launch(path, 128, 2)
+    gpu.step(1)
+    orc.step(1)
+    assert rel_err(gpu.populations(), orc.populations()) < TOL
+    for k in range(2 if path == "several" else 1):
+        hg, ho = gpu.history(0, 1, body=k), orc.history(0, 1, body=k)
+        # sums of some hundred terms of the populations' size
+        assert rel_err(hg[:, 1:4], ho[:, 1:4]) < 1e-10 and rel_err(hg[:, 12:15], ho[:, 12:15]) < 1e-10
+    gpu.close()
+
+
+@pytest.mark.parametrize("eta", [1.2e-10, 1.1e-10, 1e-20])
+def test_allocation_free_step_at_the_smallest_eta(eta):
+    import torch
+    import paper_1905_05110_gb300 as vp
+    from test_zz_no_alloc import _caller_buffers, _problem, _state_bytes, _stored_to_full
+    p = dict(_problem("disk"), eta=eta)
+    gpu, orc = make_pair(p, "f64", hist_cap=8)
+    dev = torch.device("cuda")
+    lat, body = vp.lattice_desc(p, "f64"), vp.body_desc(p["body"])
+    sizes, pops, state = _caller_buffers(lat, body, 8, dev)
+    src = gpu._tensors["f0"]
+    off = (-src.data_ptr()) % 256
+    pops[0].copy_(src[off:off + int(sizes.populations)])
+    sb = _state_bytes(p["body"])
+    state[:sb.size].copy_(torch.from_numpy(sb))
+    vp.vplbm_step_noalloc(lat, body, [t.data_ptr() for t in pops], state.data_ptr(), None, 8, 1,
+                          torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    orc.step(1)
+    raw = pops[1].cpu().numpy().view(np.float64)
+    assert rel_err(_stored_to_full(raw, p["nx"], p["ny"], "f64"), orc.populations()) < TOL
+    gpu.close()
