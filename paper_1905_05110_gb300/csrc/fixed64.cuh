@@ -495,7 +495,8 @@ VPLBM_FX bool fx_moments_dev(const FixedConsts &k, const float d[9], double &rho
 // Equilibrium (Eq. 11) of (rho, u): val[a] in units of 2^(E - 62) for the
 // deviation f_a - w_a rho0 (dev), of 2^(E - 59) for the full f_a.  False if
 // out of range (|u| >= 1/4, rho outside [rho0 / 2, 1.5 2^E); dev: a density
-// further than 2^(E - 4) from rho0).
+// further than 2^(E - 4) from rho0, a deviation of w_a 2^(E + 1) or more,
+// which its finer unit does not hold: |u| above 0.2 along a diagonal).
 VPLBM_FX bool fx_equilibrium(const FixedConsts &k, uint64_t rho_b, uint64_t ux_b, uint64_t uy_b, bool dev, long long val[9])
 {
     const uint32_t rh = (uint32_t)(rho_b >> 32), xh = (uint32_t)(ux_b >> 32) & 0x7fffffffu, yh = (uint32_t)(uy_b >> 32) & 0x7fffffffu;
@@ -522,7 +523,13 @@ VPLBM_FX bool fx_equilibrium(const FixedConsts &k, uint64_t rho_b, uint64_t ux_b
         const long long poly = ((3 * cu) >> 1) + 18 * cu2 - u15;   // 3 c.u + 9/2 (c.u)^2 - 3/2 u^2, 2^60
         const long long rp = fx_mul(r8, fx_split(2 * poly));        // rho poly, 2^(E - 59)
         const FxFactor w = a == 0 ? k.w0 : a <= 4 ? k.w1 : k.w2;    // w_a / 2^0, 4/9 < 1/2
-        val[a] = dev ? fx_mul((drho + rp) * 8, w) : fx_mul(rho + rp, w);
+        if (dev) {
+            const long long d = drho + rp;
+            if ((uint64_t)(d + (1LL << 60)) >= (uint64_t)(1LL << 61)) return false;
+            val[a] = fx_mul(8 * d, w);
+        } else {
+            val[a] = fx_mul(rho + rp, w);
+        }
     }
     return true;
 }

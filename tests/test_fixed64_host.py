@@ -36,6 +36,19 @@ extern "C" int fx_host_update(const double *s, double rho0, double gx, double gy
     }
     return k.ok;
 }
+
+// n nodes (rho, ux, uy): the equilibrium's populations, or (dev) their deviations from w rho0
+extern "C" void fx_host_equilibrium(double rho0, int dev, long n, const double *m, double *out, int *done)
+{
+    const double s[9] = {1, 1, 1, 1, 1, 1, 1, 1, 1};
+    FixedConsts k;
+    fold_fixed(k, s, rho0, 0.0, 0.0, 0.0);
+    for (long q = 0; q < n; ++q) {
+        long long v[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
+        done[q] = k.ok && fx_equilibrium(k, fx_bits(m[3 * q]), fx_bits(m[3 * q + 1]), fx_bits(m[3 * q + 2]), dev != 0, v);
+        for (int a = 0; a < 9; ++a) out[9 * q + a] = ldexp((double)v[a], k.e - (dev ? 62 : 59));
+    }
+}
 """
 
 M = np.array([[1, 1, 1, 1, 1, 1, 1, 1, 1], [-4, -1, -1, -1, -1, 2, 2, 2, 2], [4, -2, -2, -2, -2, 1, 1, 1, 1],
@@ -130,3 +143,23 @@ def test_rates_at_the_ends_of_their_range(host, rates, g, eta):
     out, _, done = _update(host, f, us, s, g=g, eta=eta)
     want, _ = _exact(f, us, s, g=g, eta=eta)
     assert np.max(np.abs(out - want)[done], initial=0.0) < UPDATE_TOL * 1.1
+
+
+@pytest.mark.parametrize("dev", [False, True])
+@pytest.mark.parametrize("rho0", [1.0, 0.99, 0.7, 0.51])
+def test_equilibrium_over_the_accepted_velocities(host, dev, rho0):
+    """All of |u_x|, |u_y| < 1/4 and densities around rho0: the right value, or left to the FP64 instructions.  FP64
+    instructions round terms of at most 4 rho about ten times."""
+    u = np.linspace(-0.2499, 0.2499, 41)
+    rho = rho0 * np.array([0.9, 0.95, 0.999, 1.0, 1.003, 1.04])
+    m = np.array([(r, x, y) for r in rho for x in u for y in u])
+    out, done = np.zeros((len(m), 9)), np.zeros(len(m), np.int32)
+    host.fx_host_equilibrium(ctypes.c_double(rho0), int(dev), ctypes.c_long(len(m)), _ptr(m), _ptr(out), _ptr(done))
+    r, ux, uy = m.T.astype(LD)
+    cu = C[0][:, None] * ux + C[1][:, None] * uy
+    w = np.array([LD(4) / 9] + [LD(1) / 9] * 4 + [LD(1) / 36] * 4)[:, None]
+    want = w * ((r - LD(rho0) if dev else r) + r * (3 * cu + LD(4.5) * cu * cu - LD(1.5) * (ux * ux + uy * uy)))
+    done = done.astype(bool)
+    near = np.abs(m[:, 0] / rho0 - 1) < 4e-3
+    assert done[near & (np.abs(m[:, 1:]).max(1) < 0.19)].all()   # a low-Mach flow stays in fixed point
+    assert np.max(np.abs(out.T - want)[:, done]) < UPDATE_TOL * 1.04 * rho0

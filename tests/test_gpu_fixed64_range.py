@@ -78,3 +78,26 @@ def test_allocation_free_step_at_the_smallest_eta(eta):
     raw = pops[1].cpu().numpy().view(np.float64)
     assert rel_err(_stored_to_full(raw, p["nx"], p["ny"], "f64"), orc.populations()) < TOL
     gpu.close()
+
+
+@pytest.mark.parametrize("precision", ["f64", "f32", "f16"])
+@pytest.mark.parametrize("rho0", [1.0, 0.99])
+def test_equilibrium_of_fast_nodes(precision, rho0):
+    """Velocities of up to 1/4 in each direction: the stored populations against FP64 arithmetic, within the rounding of
+    the storage (half a unit of the deviation; FP16: of its smallest step too)."""
+    import paper_1905_05110_gb300 as vp
+    v = np.array([-0.249, -0.22, -0.19, -0.1, 0.0, 0.1, 0.19, 0.22, 0.249])
+    ux, uy = np.meshgrid(v, v)
+    rho = rho0 * (1 + 0.01 * np.random.default_rng(4).uniform(-1, 1, ux.shape))
+    p = wl.periodic_box(9, 9)
+    p["rho0"] = rho0
+    sim = vp.Simulation(p, precision, history_capacity=4)
+    sim.init_equilibrium(rho, ux, uy)
+    w = np.array([4 / 9] + [1 / 9] * 4 + [1 / 36] * 4)[:, None, None]
+    c = np.array([[0, 0], [1, 0], [0, 1], [-1, 0], [0, -1], [1, 1], [-1, 1], [-1, -1], [1, -1]], dtype=float)
+    cu = c[:, 0, None, None] * ux + c[:, 1, None, None] * uy
+    feq = w * rho * (1 + 3 * cu + 4.5 * cu * cu - 1.5 * (ux * ux + uy * uy))
+    unit = {"f64": 0.0, "f32": 2.0 ** -24, "f16": 2.0 ** -11}[precision]
+    err = np.abs(sim.populations() - feq) - unit * np.abs(feq - w * rho0)
+    assert np.max(err) < TOL + (6e-8 if precision == "f16" else 0)
+    sim.close()
