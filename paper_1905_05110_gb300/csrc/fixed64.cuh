@@ -396,12 +396,16 @@ VPLBM_FX double fx_signed_to(long long x, int k)
 }
 
 // x 2^k as a float, to nearest, for |x| < 2^62 and a result in the normal
-// range (or zero).  near_tie is set where x is within 512 units of halfway
-// between two floats: FP64 arithmetic, whose error is below that, could round
-// the other way there.
+// range.  near_tie is set where x is within 512 units of halfway between two
+// floats (FP64 arithmetic, whose error is below that, could round the other
+// way there), and where x is too small for the float's digits or zero (what
+// was rounded to zero need not be).
 VPLBM_FX float fx_signed_to_float(long long x, int k, bool &near_tie)
 {
-    if (x == 0) return 0.f;
+    if (x == 0) {
+        near_tie = true;
+        return 0.f;
+    }
     const uint64_t m = x < 0 ? 0 - (uint64_t)x : (uint64_t)x;
     const uint32_t hi = (uint32_t)(m >> 32);
     const int n = hi ? fx_clz(hi) : 32 + fx_clz((uint32_t)m);

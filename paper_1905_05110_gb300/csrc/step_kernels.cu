@@ -83,6 +83,11 @@ __global__ void init_equilibrium_kernel(const StepParams p, const double *rho_f,
     const double ux = ux_f ? ux_f[k] : 0.0;
     const double uy = uy_f ? uy_f[k] : 0.0;
     S *fout = static_cast<S *>(p.fout);
+    if (Prec<P>::DEV && rho == p.rho0 && ux == 0.0 && uy == 0.0) {   // at rest: no deviation
+#pragma unroll
+        for (int a = 0; a < NQ; ++a) stv(fout + a * p.ps + k, (typename Prec<P>::T)0);
+        return;
+    }
     long long val[NQ];
     if (p.fx.ok && fx_equilibrium(p.fx, (uint64_t)__double_as_longlong(rho), (uint64_t)__double_as_longlong(ux),
                                   (uint64_t)__double_as_longlong(uy), Prec<P>::DEV, val)) {

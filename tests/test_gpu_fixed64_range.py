@@ -101,3 +101,21 @@ def test_equilibrium_of_fast_nodes(precision, rho0):
     err = np.abs(sim.populations() - feq) - unit * np.abs(feq - w * rho0)
     assert np.max(err) < TOL + (6e-8 if precision == "f16" else 0)
     sim.close()
+
+
+@pytest.mark.parametrize("u", [1e-6, 1e-15, 1e-20, 1e-28])
+def test_equilibrium_of_slow_nodes(u):
+    """FP32 storage keeps the relative precision of any velocity: half a unit of each stored deviation."""
+    import paper_1905_05110_gb300 as vp
+    p = wl.periodic_box(8, 6)
+    sim = vp.Simulation(p, "f32", history_capacity=4)
+    sim.init_equilibrium(None, u, -0.5 * u)
+    c = np.array([[0, 0], [1, 0], [0, 1], [-1, 0], [0, -1], [1, 1], [-1, 1], [-1, -1], [1, -1]], dtype=float)
+    w = np.array([4 / 9] + [1 / 9] * 4 + [1 / 36] * 4)
+    cu, u2 = c @ np.array([u, -0.5 * u]), 1.25 * u * u
+    want = w * (3 * cu + 4.5 * cu * cu - 1.5 * u2)
+    off = (-sim._tensors["f0"].data_ptr()) % 256
+    ps = (8 * 6 + 127) // 128 * 128
+    got = sim._tensors["f0"][off:off + 9 * ps * 4].cpu().numpy().view(np.float32).reshape(9, ps)[:, :48].astype(float)
+    assert np.all(np.abs(got - want[:, None]) <= 1.01 * 2.0 ** -24 * np.abs(want[:, None]) + 1e-45)
+    sim.close()
