@@ -120,6 +120,12 @@ VPLBM_FX int fx_clz(uint32_t x)
 #endif
 }
 
+VPLBM_FX int fx_clz64(uint64_t x)
+{
+    const uint32_t hi = (uint32_t)(x >> 32);
+    return hi ? fx_clz(hi) : 32 + fx_clz((uint32_t)x);
+}
+
 VPLBM_FX uint64_t fx_bits(double d)
 {
 #if defined(__CUDA_ARCH__)
@@ -388,8 +394,7 @@ VPLBM_FX double fx_signed_to(long long x, int k)
 {
     if (x == 0) return 0.0;
     const uint64_t sign = (uint64_t)x & 0x8000000000000000ull, m = x < 0 ? 0 - (uint64_t)x : (uint64_t)x;
-    const uint32_t hi = (uint32_t)(m >> 32);
-    const int n = hi ? fx_clz(hi) : 32 + fx_clz((uint32_t)m);
+    const int n = fx_clz64(m);
     const uint64_t y = m << n;   // leading bit at 63
     const uint64_t q = y >> 11, half = (y >> 10) & 1, rest = (y & 0x3ff) | (q & 1);
     return fx_double(sign | ((q + (half & (rest != 0))) + ((uint64_t)(1023 + 63 - 1 + k - n) << 52)));
@@ -407,23 +412,13 @@ VPLBM_FX float fx_signed_to_float(long long x, int k, bool &near_tie)
         return 0.f;
     }
     const uint64_t m = x < 0 ? 0 - (uint64_t)x : (uint64_t)x;
-    const uint32_t hi = (uint32_t)(m >> 32);
-    const int n = hi ? fx_clz(hi) : 32 + fx_clz((uint32_t)m);
+    const int n = fx_clz64(m);
     const uint64_t y = m << n;
     const long long off = (long long)(y & 0xffffffffffull) - (1LL << 39);   // from halfway
     near_tie = near_tie || n >= 30 || (off < 0 ? -off : off) <= (512LL << n);
     const uint32_t t = (uint32_t)(y >> 32) | ((uint32_t)y != 0);   // the leading 32 bits, the rest sticky
     const float f = (float)t * fx_pow2f(k + 32 - n);
     return x < 0 ? -f : f;
-}
-
-// A float of magnitude below 2^(E - 3) in units of 2^(E - 62) (truncated).
-VPLBM_FX long long fx_from_float(uint32_t b, int e)
-{
-    const uint32_t m = (b & 0x7fffffu) | 0x800000u, ex = (b >> 23) & 0xffu;
-    const uint32_t s = (uint32_t)(123 + e) - ex;
-    const uint64_t x = ((uint64_t)m << 35) >> (s < 63 ? s : 63);
-    return (b >> 31) ? -(long long)x : (long long)x;
 }
 
 // A double of magnitude below 1/4 times 2^61, to nearest even.
@@ -438,8 +433,7 @@ VPLBM_FX long long fx_from_signed(uint64_t b)
 }
 
 // rho and u of nine pulled populations away from the body, without a uniform
-// acceleration: FP64 storage, and FP32 / FP16 storage (deviations, as floats).
-// False if the node is out of range.
+// acceleration: FP64 storage.  False if the node is out of range.
 VPLBM_FX bool fx_moments(const FixedConsts &k, const uint64_t fb[9], double &rho_o, double &ux_o, double &uy_o)
 {
     uint32_t top = 0, low = 0xffffffffu;
@@ -468,31 +462,52 @@ VPLBM_FX bool fx_moments(const FixedConsts &k, const uint64_t fb[9], double &rho
     return true;
 }
 
+// The same for FP32 / FP16 storage (deviations, as floats).  A deviation has
+// its 24 bits relative to itself, so the sums are on a grid of their own, set
+// by the node's largest one: d 2^(58 - T), 2^T > |d|, on which a float down to
+// 2^-34 of the largest is exact (a node with a smaller one that is not zero,
+// or with a largest one below 2^-92, is left to the FP64 code).  The sums are
+// then exact, and u has the precision of a double for any size of the
+// deviations; on the grid of rho0 a deviation of 1e-14 would keep 15 bits.
 VPLBM_FX bool fx_moments_dev(const FixedConsts &k, const float d[9], double &rho_o, double &ux_o, double &uy_o)
 {
-    uint32_t top = 0;
+    uint32_t top = 0, low = 0xffffffffu;   // largest; smallest but zero, minus one
     long long f[9];
 #if defined(__CUDA_ARCH__)
 #pragma unroll
 #endif
     for (int a = 0; a < 9; ++a) {
-        const uint32_t b = fx_float_bits(d[a]), m = b & 0x7fffffffu;
+        const uint32_t m = fx_float_bits(d[a]) & 0x7fffffffu;
         top = m > top ? m : top;
-        f[a] = fx_from_float(b, k.e);
+        low = m - 1u < low ? m - 1u : low;
     }
-    if (k.e < -30 || k.e > 60 || top >= (uint32_t)(124 + k.e) << 23) return false;
+    const int et = (int)(top >> 23), el = (int)((low + 1u) >> 23);
+    if (k.e < -30 || k.e > 60 || top >= (uint32_t)(124 + k.e) << 23 || (top != 0 && (et < 35 || et - el > 34))) return false;
+#if defined(__CUDA_ARCH__)
+#pragma unroll
+#endif
+    for (int a = 0; a < 9; ++a) {
+        const uint32_t b = fx_float_bits(d[a]), s = (uint32_t)et - ((b >> 23) & 0xffu);
+        const long long x = s > 34 || top == 0 ? 0 : (long long)(((uint64_t)((b & 0x7fffffu) | 0x800000u) << 34) >> s);
+        f[a] = (b >> 31) ? -x : x;
+    }
     const long long sx = f[5] - f[6] - f[7] + f[8], sy = f[5] + f[6] - f[7] - f[8];
-    const long long rs = f[0] + f[1] + f[2] + f[3] + f[4] + f[5] + f[6] + f[7] + f[8];
-    const long long jx = f[1] - f[3] + sx, jy = f[2] - f[4] + sy;
-    const long long rho = k.rho0 + ((rs + 4) >> 3);
-    constexpr long long J = 1LL << 59;   // |j| < 1/8: j << 3 below stays in 62 bits
-    if ((uint64_t)(rho - (1LL << 58)) >= (uint64_t)(1LL << 59) || (uint64_t)(jx + J) >= (uint64_t)(2 * J) ||
-        (uint64_t)(jy + J) >= (uint64_t)(2 * J))
-        return false;
+    const long long rs = f[0] + f[1] + f[2] + f[3] + f[4] + f[5] + f[6] + f[7] + f[8];   // below 9 2^58
+    const long long jx = f[1] - f[3] + sx, jy = f[2] - f[4] + sy;                        // below 6 2^58
+    const int T = et - 126, n = k.e - 1 - T;   // to the grid of rho: 2^(E - 59); n >= 2
+    const long long rho = k.rho0 + (n > 62 ? 0 : (rs + (1LL << (n - 1))) >> n);
+    if ((uint64_t)(rho - (1LL << 58)) >= (uint64_t)(1LL << 59)) return false;
     const FxFactor inv = fx_split(fx_recip(rho));   // 2^120 / rho
+    auto quotient = [&](long long j) {              // its leading bit to bit 61 first
+        if (j == 0) return 0.0;
+        const uint64_t m = j < 0 ? 0 - (uint64_t)j : (uint64_t)j;
+        const int up = fx_clz64(m) - 2;
+        const long long q = fx_mul((long long)(m << up), inv);
+        return fx_signed_to(j < 0 ? -q : q, T - k.e - 55 - up);
+    };
     rho_o = fx_to(rho, k.e);
-    ux_o = fx_signed_to(fx_mul((long long)((uint64_t)jx << 3), inv), -62);
-    uy_o = fx_signed_to(fx_mul((long long)((uint64_t)jy << 3), inv), -62);
+    ux_o = quotient(jx);
+    uy_o = quotient(jy);
     return true;
 }
 

@@ -64,6 +64,15 @@ extern "C" void fx_host_equilibrium_f32(double rho0, long n, const double *m, fl
         done[q] = done[q] && !near_tie;
     }
 }
+
+// n nodes of deviations d[9]: rho, u_x, u_y
+extern "C" void fx_host_moments_dev(double rho0, long n, const float *d, double *out, int *done)
+{
+    const double s[9] = {1, 1, 1, 1, 1, 1, 1, 1, 1};
+    FixedConsts k;
+    fold_fixed(k, s, rho0, 0.0, 0.0, 0.0);
+    for (long q = 0; q < n; ++q) done[q] = k.ok && fx_moments_dev(k, d + 9 * q, out[3 * q], out[3 * q + 1], out[3 * q + 2]);
+}
 """
 
 M = np.array([[1, 1, 1, 1, 1, 1, 1, 1, 1], [-4, -1, -1, -1, -1, 2, 2, 2, 2], [4, -2, -2, -2, -2, 1, 1, 1, 1],
@@ -197,3 +206,41 @@ def test_equilibrium_deviations_of_slow_nodes(host):
     done = done.astype(bool)
     assert done[np.abs(u).max(1) > 1e-3].mean() > 0.98   # a flow at speed stays in fixed point
     assert np.array_equal(out.T[:, done], want.astype(np.float32)[:, done])
+
+
+@pytest.mark.parametrize("rho0", [1.0, 0.7, 0.51])
+@pytest.mark.parametrize("spread", [0, 3, 9, 30])
+def test_fields_of_deviations_of_any_size(host, rho0, spread):
+    """rho and u of FP32 / FP16 storage: a deviation has its 24 bits whatever its size, so u has the precision of a double
+    (2^-53 for the rounding, 2^-56 for the quotient), or the node is left to the FP64 instructions."""
+    rng = np.random.default_rng(8)
+    n = 20000
+    size = 10.0 ** rng.uniform(-30, -1.3, n)
+    d = (size[:, None] * 10.0 ** -rng.uniform(0, spread, (n, 9)) * rng.uniform(-1, 1, (n, 9))).astype(np.float32)
+    d[rng.uniform(size=(n, 9)) < 0.05] = 0
+    d[::50] = 0                                     # at rest
+    d[1::50, 3], d[1::50, 1] = d[1::50, 1], d[1::50, 1] * np.float32(1 + 2.0 ** -20)   # the sums cancel
+    d[1::50, 5:] = 0
+    d = np.ascontiguousarray(d)
+    out, done = np.zeros((n, 3)), np.zeros(n, np.int32)
+    host.fx_host_moments_dev(ctypes.c_double(rho0), ctypes.c_long(n), _ptr(d), _ptr(out), _ptr(done))
+    done = done.astype(bool)
+    f = d.T.astype(LD)
+    jx, jy = f[1] - f[3] + (f[5] - f[6]) + (f[8] - f[7]), f[2] - f[4] + (f[5] + f[6]) - (f[7] + f[8])
+    rho = LD(rho0) + f.sum(0)
+    for got, want in zip(out.T, (rho, jx / rho, jy / rho)):
+        assert np.all(np.abs(got - want)[done] <= 1.3e-16 * np.abs(want)[done])
+    inside = (size > 1e-25) & (rho > 0.5)           # the density's range is [2^(E-1), 1.5 2^E)
+    if spread < 9:                                  # nearly all within 2^34 of the node's largest
+        assert done[inside].mean() > 0.999
+    rest = out[::50][done[::50]]
+    assert np.all(rest == [rho0, 0.0, 0.0])
+
+
+@pytest.mark.parametrize("value", [np.nan, np.inf, -np.inf, 0.2, 1e-42])
+def test_fields_of_deviations_out_of_range_are_left_to_fp64(host, value):
+    d = np.full((9, 9), 1e-3, np.float32)
+    d[np.arange(9), np.arange(9)] = value
+    out, done = np.zeros((9, 3)), np.ones(9, np.int32)
+    host.fx_host_moments_dev(ctypes.c_double(1.0), ctypes.c_long(9), _ptr(d), _ptr(out), _ptr(done))
+    assert not done.any()

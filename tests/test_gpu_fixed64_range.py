@@ -119,3 +119,28 @@ def test_equilibrium_of_slow_nodes(u):
     got = sim._tensors["f0"][off:off + 9 * ps * 4].cpu().numpy().view(np.float32).reshape(9, ps)[:, :48].astype(float)
     assert np.all(np.abs(got - want[:, None]) <= 1.01 * 2.0 ** -24 * np.abs(want[:, None]) + 1e-45)
     sim.close()
+
+
+@pytest.mark.parametrize("precision,u", [("f32", 0.05), ("f32", 1e-9), ("f32", 1e-14), ("f32", 1e-25), ("f16", 0.05), ("f16", 1e-3)])
+def test_fields_of_a_slow_flow(precision, u):
+    """u of FP32 / FP16 storage against the stored deviations' own sums, for a flow of any speed: FP64 rounding."""
+    import paper_1905_05110_gb300 as vp
+    nx, ny = 40, 32
+    p = wl.periodic_box(nx, ny)
+    sim = vp.Simulation(p, precision, history_capacity=4)
+    rng = np.random.default_rng(9)
+    ux, uy = u * rng.uniform(-1, 1, (2, ny, nx))
+    sim.init_equilibrium(None, ux, uy)
+    off = (-sim._tensors["f0"].data_ptr()) % 256
+    ps = (nx * ny + 127) // 128 * 128
+    dt = np.float32 if precision == "f32" else np.float16
+    raw = sim._tensors["f0"][off:off + 9 * ps * dt().nbytes].cpu().numpy().view(dt)
+    d = raw.reshape(9, ps)[:, :nx * ny].reshape(9, ny, nx).astype(np.longdouble)
+    c = [(0, 0), (1, 0), (0, 1), (-1, 0), (0, -1), (1, 1), (-1, 1), (-1, -1), (1, -1)]
+    d = np.array([np.roll(d[a], (c[a][1], c[a][0]), (0, 1)) for a in range(9)])   # the pulled ones
+    rho = 1 + d.sum(0)
+    got = sim.fields()
+    want = (rho, sum(c[a][0] * d[a] for a in range(9)) / rho, sum(c[a][1] * d[a] for a in range(9)) / rho)
+    for g, w in zip(got, want):
+        assert np.max(np.abs(g - w)) < 1e-15 * np.max(np.abs(w))
+    sim.close()
