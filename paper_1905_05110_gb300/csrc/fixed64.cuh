@@ -23,7 +23,8 @@
 //
 // Measured (GB300, us per step, best block shape): 2048 x 1024 513 -> 63.5
 // (32.9 k MLUPS, 4.7 TB/s), 256 x 128 28 -> 13.5 (there the launch boundary
-// and the body's sums remain).
+// and the body's sums remain); 2048 x 1024 under a uniform
+// acceleration 114.
 //
 // Range.  A node takes this path if every population is in
 // [2^(E-32), 2^E), rho in [2^(E-1), 1.5 2^E), |j| < 0.35 2^E and (body
@@ -62,7 +63,11 @@ struct FixedConsts {
     // forcing: (1 - s/2) / 6 for e and eps, / 12 for q, / 2 and / 4 for the
     // stress, 1/6, and pen_k / 8 (pen_k = 1 / (eta + 1/2) tends to 2)
     FxFactor h1, h2, h4, h6, h7, h8, sixth, k8;
-    long long gvx, gvy;         // g 2^60
+    long long gvx, gvy;         // g 2^60, for the velocity j / rho + g / 2
+    // g / 16 for the force rho g: two digits (2^-64) would put it off by up to
+    // 4e-19, every step with the same sign
+    FxFactor gx, gy;
+    int gx3, gy3;               // its third digits (2^-96)
     int forced;                 // g is not zero
     long long rho0;             // in units of 2^(E - 59)
     FxFactor w0, w1, w2;        // the weights
@@ -80,6 +85,19 @@ inline FxFactor fx_factor(double r, int &ok)
     f.lo = (int)(uint32_t)(uint64_t)v;
     f.hi = (int)((v - (long long)f.lo) >> 32);
     return f;
+}
+
+// g / 16 and its third digit.  other: the other component.  A force of a few
+// units or less is not rounded without a bias (a uniform density rounds it the
+// same way everywhere): below 2^-40 the run takes the FP64 instructions, but
+// for a component that is only the other's rounding (a direction at right
+// angles computed by cos).
+inline FxFactor fx_accel(double g, double other, int &third, int &ok)
+{
+    if (g != 0.0 && fabs(g) < 0x1p-40 && !(fabs(g) <= 0x1p-50 * fabs(other))) ok = 0;
+    const double r = g / 16.0, rest = ldexp(r, 64) - rint(ldexp(r, 64));   // both exact, or below 2^-96
+    third = (int)fmin(rint(ldexp(rest, 32)), 2147483647.0);
+    return fx_factor(r, ok);
 }
 
 inline void fold_fixed(FixedConsts &k, const double *s, double rho0, double gx, double gy, double pen_k)
@@ -105,6 +123,8 @@ inline void fold_fixed(FixedConsts &k, const double *s, double rho0, double gx, 
     k.k8 = fx_factor(0.125 * pen_k, ok);
     k.gvx = llrint(ldexp(gx, 60));
     k.gvy = llrint(ldexp(gy, 60));
+    k.gx = fx_accel(gx, gy, k.gx3, ok);
+    k.gy = fx_accel(gy, gx, k.gy3, ok);
     k.forced = gx != 0.0 || gy != 0.0;
     k.rho0 = llrint(ldexp(rho0, 59 - e));
     k.w0 = fx_factor(4.0 / 9.0, ok); k.w1 = fx_factor(1.0 / 9.0, ok); k.w2 = fx_factor(1.0 / 36.0, ok);
@@ -189,6 +209,14 @@ VPLBM_FX long long fx_mul(long long x, FxFactor r)
     return (long long)a.hi * r.hi + (m >> 32);
 }
 
+// The same with a third digit (2^-96) of r.
+VPLBM_FX long long fx_mul3(long long x, FxFactor r, int third)
+{
+    const FxFactor a = fx_split(x);
+    const long long m = (long long)a.lo * r.hi + 0x80000000LL + (long long)a.hi * r.lo + (((long long)a.hi * third) >> 32);
+    return (long long)a.hi * r.hi + (m >> 32);
+}
+
 // The double with bits b, in [2^(E-32), 2^E), on the grid (truncated).
 VPLBM_FX long long fx_from(uint64_t b, int e)
 {
@@ -249,13 +277,16 @@ VPLBM_FX long long fx_recip(long long rho)
 // acceleration) does differently, a function of its own on the device: few
 // nodes take it, and inlined it costs the others registers.  In: the moments
 // (v: velocity times 2^61) and the solid velocity us; out: the increments
-// along the rows of M and G / 6, and a 2^60 of the penalization.  False if
-// the slip is out of range.
+// along the rows of M, G / 6, what an axis population takes beside that under
+// a uniform acceleration (r), and a 2^60 of the penalization.  False if the
+// slip is out of range.
 struct FxForced {
     long long rho, jx, jy, vx, vy, usx, usy, f0, sa, sd, qx, qy, pxx, pxy;   // in
-    long long de, dep, dqx, dqy, dp, dr, gx6, gy6, ax, ay;                   // out
+    long long de, dep, dqx, dqy, dp, dr, gx6, gy6, rx, ry, ax, ay;           // out
 };
 
+// G: the lattice may be under a uniform acceleration.
+template <bool G>
 VPLBM_FX bool fx_forced_here(const FixedConsts &k, bool chi, FxForced &w)
 {
     const long long wx = w.vx + k.gvx, wy = w.vy + k.gvy;   // v = j / rho + g / 2
@@ -269,7 +300,28 @@ VPLBM_FX bool fx_forced_here(const FixedConsts &k, bool chi, FxForced &w)
     }
     const FxFactor ux = fx_split(wx + ax), uy = fx_split(wy + ay);   // u = v + a / 2
     const long long r8 = (long long)((uint64_t)w.rho << 3);
-    const long long Gx = fx_mul(r8, fx_split(2 * (ax + k.gvx))), Gy = fx_mul(r8, fx_split(2 * (ay + k.gvy)));
+    long long Gx, Gy;   // rho (a + g)
+    if (!G || !k.forced) {
+        Gx = fx_mul(r8, fx_split(2 * ax));
+        Gy = fx_mul(r8, fx_split(2 * ay));
+        w.gx6 = fx_mul(Gx, k.sixth);
+        w.gy6 = fx_mul(Gy, k.sixth);
+    } else {
+        // half of it is rounded, and what the four diagonal populations do not
+        // take of a sixth each goes to the other two: the node gains Gx, while
+        // six roundings of Gx / 6 favour the sign of g by half a unit
+        long long hx = fx_mul3(r8, k.gx, k.gx3), hy = fx_mul3(r8, k.gy, k.gy3);
+        if (chi) {
+            hx += fx_mul(r8, fx_split(ax));
+            hy += fx_mul(r8, fx_split(ay));
+        }
+        Gx = 2 * hx;
+        Gy = 2 * hy;
+        w.gx6 = fx_mul(Gx, k.sixth);
+        w.gy6 = fx_mul(Gy, k.sixth);
+        w.rx = hx - 3 * w.gx6;
+        w.ry = hy - 3 * w.gy6;
+    }
     const long long mx = w.jx + (Gx >> 1), my = w.jy + (Gy >> 1);    // rho u = j + G / 2
     const long long mx8 = (long long)((uint64_t)mx << 3), my8 = (long long)((uint64_t)my << 3);
     const long long A = fx_mul(mx8, ux), B = fx_mul(my8, uy), C = fx_mul(mx8, uy);
@@ -282,8 +334,6 @@ VPLBM_FX bool fx_forced_here(const FixedConsts &k, bool chi, FxForced &w)
     w.dqy = fx_mul(w.qy - (Gy >> 1), k.r6) - fx_mul(Gy, k.h6);
     w.dp = fx_mul(A - B - w.pxx, k.r7) + fx_mul(xx - yy, k.h7);
     w.dr = fx_mul(C - w.pxy, k.r8) + fx_mul(xy, k.h8);
-    w.gx6 = fx_mul(Gx, k.sixth);
-    w.gy6 = fx_mul(Gy, k.sixth);
     w.ax = ax;
     w.ay = ay;
     return true;
@@ -294,13 +344,14 @@ __device__ __noinline__
 #else
 inline
 #endif
-bool fx_forced(const FixedConsts &k, bool chi, FxForced &w) { return fx_forced_here(k, chi, w); }
+bool fx_forced(const FixedConsts &k, bool chi, FxForced &w) { return fx_forced_here<true>(k, chi, w); }
 
 // One node: pulled populations f (bits of doubles) -> post-collision
 // populations out.  chi: the node is in a body of solid velocity us (times
 // 2^61).  Returns false (out untouched) if the node is out of range; rho and
 // a 2^60 (the penalization's acceleration) are kept for the body's sums.
-// HERE: a caller of solid nodes only has the penalized part inlined.
+// HERE: a caller of solid nodes only, without a uniform acceleration, has the
+// penalized part inlined.
 template <bool HERE = false>
 #if defined(__CUDACC__)
 __device__ __forceinline__
@@ -339,9 +390,15 @@ bool fx_update(const FixedConsts &k, const uint64_t fb[9], bool chi, long long u
         FxForced w;
         w.rho = rho; w.jx = jx; w.jy = jy; w.vx = vx; w.vy = vy; w.usx = usx; w.usy = usy;
         w.f0 = f[0]; w.sa = sa; w.sd = sd; w.qx = dqx; w.qy = dqy; w.pxx = b13 - b24; w.pxy = d56 - d87;
-        if (!(HERE ? fx_forced_here(k, chi, w) : fx_forced(k, chi, w))) return false;
+        if (!(HERE ? fx_forced_here<false>(k, chi, w) : fx_forced(k, chi, w))) return false;
         de = w.de; dep = w.dep; dqx = w.dqx; dqy = w.dqy; dp = w.dp; dr = w.dr;
         gx6 = w.gx6; gy6 = w.gy6;
+        if (!HERE && k.forced) {
+            f[1] += w.rx;
+            f[3] -= w.rx;
+            f[2] += w.ry;
+            f[4] -= w.ry;
+        }
         ax_o = w.ax;
         ay_o = w.ay;
     } else {

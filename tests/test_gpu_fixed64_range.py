@@ -144,3 +144,25 @@ def test_fields_of_a_slow_flow(precision, u):
     for g, w in zip(got, want):
         assert np.max(np.abs(g - w)) < 1e-15 * np.max(np.abs(w))
     sim.close()
+
+
+@pytest.mark.parametrize("kernel", ["scalar", "resident"])
+@pytest.mark.parametrize("g", [(1e-9, -2e-9), (1e-12, 0.0), (3e-14, 1e-15)])
+def test_momentum_gained_from_a_uniform_acceleration(kernel, g):
+    """FP64 storage, periodic: rho g per node and step.  Tolerance: five deviations of the mean of n roundings of at most
+    1e-17 rho a node and step (doubles of 2^-57 and 2^-59, half a unit each)."""
+    import paper_1905_05110_gb300 as vp
+    nx, ny, steps = 67, 45, 100
+    p = wl.periodic_box(nx, ny, tau=0.7, g_fluid=g)
+    sim = vp.Simulation(p, "f64", history_capacity=4)
+    sim.set_launch(kernel, 128, 2)
+    sim.set_populations(wl.random_populations(nx, ny, seed=11, amp=0.03))
+    c = np.array([[0, 1, 0, -1, 0, 1, -1, -1, 1], [0, 0, 1, 0, -1, 1, 1, -1, -1]])
+    f0 = sim.populations().astype(np.longdouble)
+    sim.step(steps)
+    f1 = sim.populations().astype(np.longdouble)
+    n = nx * ny * steps
+    gain = np.tensordot(c, f1 - f0, axes=(1, 0)).sum(axis=(1, 2)) / n
+    mean_rho = f0.sum() / (nx * ny)
+    assert np.max(np.abs(gain - mean_rho * np.array(g))) < 5 * 1e-17 / np.sqrt(n)
+    sim.close()
