@@ -316,14 +316,14 @@ vplbm_status vplbm_get_body_k(vplbm_ctx *ctx, int k, double q[3], double v[3], l
  *                          storage, at most one body, a lattice of at most
  *                          about 530 000 nodes (FP32) or 150 000 (FP64)):
  *                          what a context of such a lattice does by default
- *                          and what vplbm_autotune may choose (vplbm_get_launch
- *                          then names the kernel of its single launches).  One cooperative
+ *                          and what vplbm_autotune may choose.  One cooperative
  *                          launch runs up to 4096 steps; the launch counts
  *                          count its steps, one VPLBM_LAUNCH_ONE_STEP each.  (block_x,
  *                          block_y): the blocks of steps that have to be
  *                          launched one by one (on a stream that is being
  *                          captured, or where a cooperative launch is
- *                          refused); 0 x 0 keeps the current ones.  Its
+ *                          refused); 0 x 0 keeps the current ones, and so
+ *                          do the blocks that vplbm_get_launch names.  Its
  *                          populations equal the scalar kernel's bit for
  *                          bit; its force sums are added in another order.
  *                          The context keeps a workspace of a few MB for it,
@@ -345,12 +345,16 @@ typedef enum {
 vplbm_status vplbm_set_launch(vplbm_ctx *ctx, int kernel, int block_x, int block_y);
 vplbm_status vplbm_get_launch(vplbm_ctx *ctx, int *kernel, int *block_x, int *block_y);
 
+/* The same of steps that are launched one by one: under the resident kernel
+ * the kernel chosen for these, otherwise what vplbm_get_launch names. */
+vplbm_status vplbm_get_step_launch(vplbm_ctx *ctx, int *kernel, int *block_x, int *block_y);
+
 /* Time every candidate kernel and block shape on the current state (the
  * state is saved and restored around the trials) and keep the fastest. */
 vplbm_status vplbm_autotune(vplbm_ctx *ctx, int steps_per_trial);
 
-/* Test hook for the bounded waits of the TMA-staged and (when chosen through
- * vplbm_set_launch) the resident kernel.  Resident: while enabled, its tiles
+/* Test hook for the bounded waits of the TMA-staged and the resident
+ * kernel.  Resident: while enabled, its tiles
  * wait in vain for the pose and give up after 20 ms; the next vplbm_sync
  * returns VPLBM_ETIMEOUT (initialise or load the state again).  TMA: when enabled,
  * the first shared-memory stage of every block waits for 16 bytes more than

@@ -25,7 +25,7 @@ __all__ = [
     "vplbm_init_equilibrium", "vplbm_set_populations", "vplbm_step", "vplbm_sync",
     "vplbm_get_populations", "vplbm_get_fields", "vplbm_get_fields_dev", "vplbm_get_history",
     "vplbm_get_body", "vplbm_create_bodies", "vplbm_get_num_bodies", "vplbm_get_history_body",
-    "vplbm_get_body_k", "MAX_BODIES", "vplbm_set_launch", "vplbm_get_launch", "vplbm_autotune",
+    "vplbm_get_body_k", "MAX_BODIES", "vplbm_set_launch", "vplbm_get_launch", "vplbm_get_step_launch", "vplbm_autotune",
     "vplbm_get_launch_count", "vplbm_get_kernel_launches", "vplbm_eval_recip_f32", "LAUNCH_KINDS", "vplbm_save", "vplbm_load", "vplbm_last_error", "vplbm_version",
     "vplbm_step_noalloc", "BodyState", "vplbm_inject_wait_timeout", "Batch",
     "vplbm_batch_create", "vplbm_batch_destroy", "vplbm_batch_member", "vplbm_batch_step",
@@ -131,6 +131,7 @@ _SIGS = {
     "vplbm_get_body_k": (C.c_int, [_CTX, C.c_int, _D, _D, C.POINTER(C.c_longlong)]),
     "vplbm_set_launch": (C.c_int, [_CTX, C.c_int, C.c_int, C.c_int]),
     "vplbm_get_launch": (C.c_int, [_CTX, C.POINTER(C.c_int), C.POINTER(C.c_int), C.POINTER(C.c_int)]),
+    "vplbm_get_step_launch": (C.c_int, [_CTX, C.POINTER(C.c_int), C.POINTER(C.c_int), C.POINTER(C.c_int)]),
     "vplbm_autotune": (C.c_int, [_CTX, C.c_int]),
     "vplbm_get_launch_count": (C.c_int, [_CTX, C.POINTER(C.c_longlong)]),
     "vplbm_get_kernel_launches": (C.c_int, [_CTX, C.POINTER(C.c_longlong)]),
@@ -392,6 +393,12 @@ def vplbm_set_launch(ctx, kernel: int, bx: int, by: int):
 def vplbm_get_launch(ctx):
     k, bx, by = C.c_int(), C.c_int(), C.c_int()
     _check(load_library().vplbm_get_launch(ctx, C.byref(k), C.byref(bx), C.byref(by)))
+    return k.value, bx.value, by.value
+
+
+def vplbm_get_step_launch(ctx):
+    k, bx, by = C.c_int(), C.c_int(), C.c_int()
+    _check(load_library().vplbm_get_step_launch(ctx, C.byref(k), C.byref(bx), C.byref(by)))
     return k.value, bx.value, by.value
 
 
@@ -658,14 +665,19 @@ class Simulation:
         vplbm_set_launch(self.ctx, k, bx, by)
 
     def launch(self):
-        """(kernel name, block_x, block_y) of the step kernel."""
+        """(kernel name, block_x, block_y) of the step kernel ("resident": the blocks of steps
+        that have to be launched one by one); set_launch takes it back."""
         k, bx, by = vplbm_get_launch(self.ctx)
         return KERNEL_NAMES[k], bx, by
 
     def autotune(self, steps_per_trial: int = 20):
-        """Time the step kernels and launch shapes over short trials, keep the fastest; returns it as launch()."""
+        """Time the step kernels and launch shapes over short trials, keep the fastest (launch() names it).
+
+        Returns (kernel name, block_x, block_y) of the fastest that is launched step by step: what
+        launch() names too, unless that is the resident kernel."""
         vplbm_autotune(self.ctx, steps_per_trial)
-        return self.launch()
+        k, bx, by = vplbm_get_step_launch(self.ctx)
+        return KERNEL_NAMES[k], bx, by
 
     @property
     def launches(self) -> int:

@@ -1191,11 +1191,12 @@ vplbm_status vplbm_set_launch(vplbm_ctx *c, int kernel, int bx, int by)
     }
     if (kernel == KERNEL_RESIDENT) {
         // (bx, by): the blocks of steps launched one by one (the 64-register
-        // FP64 or 40-register FP32 kernel); 0 x 0 keeps the current choice
+        // FP64 or 40-register FP32 kernel); 0 x 0 or the blocks in use keep
+        // the current choice, so that what vplbm_get_launch named is kept
         if (!c->res_ok)
             return fail(VPLBM_EUNSUPPORTED, "the resident kernel needs FP32 or FP64 storage, one body and a lattice that fits shared memory");
         const int k0 = step_kernel(c);
-        if (bx != 0 || by != 0) {
+        if ((bx != 0 || by != 0) && (bx != c->bx || by != c->by)) {
             const int was = c->kernel;
             c->kernel = k0;
             const vplbm_status st = vplbm_set_launch(c, c->precision == VPLBM_F64 ? KERNEL_SCALAR : KERNEL_SCALAR_40, bx, by);
@@ -1208,7 +1209,6 @@ vplbm_status vplbm_set_launch(vplbm_ctx *c, int kernel, int bx, int by)
             c->base_kernel = k0;
         }
         c->kernel = KERNEL_RESIDENT;
-        c->res_chosen = true;
         return VPLBM_OK;
     }
     if (kernel == KERNEL_FUSED2) {
@@ -1257,18 +1257,23 @@ vplbm_status vplbm_set_launch(vplbm_ctx *c, int kernel, int bx, int by)
 vplbm_status vplbm_get_launch(vplbm_ctx *c, int *kernel, int *bx, int *by)
 {
     if (!c) return fail(VPLBM_EINVAL, "context is NULL");
-    // the resident kernel is named where it was asked for; a default or tuned
-    // context names the kernel of its steps that are launched one by one
-    if (kernel) *kernel = c->res_chosen ? c->kernel : step_kernel(c);
+    if (kernel) *kernel = c->kernel;
     if (bx) *bx = c->bx;
     if (by) *by = c->by;
     return VPLBM_OK;
 }
 
+vplbm_status vplbm_get_step_launch(vplbm_ctx *c, int *kernel, int *bx, int *by)
+{
+    const vplbm_status st = vplbm_get_launch(c, kernel, bx, by);
+    if (st == VPLBM_OK && kernel) *kernel = step_kernel(c);
+    return st;
+}
+
 vplbm_status vplbm_inject_wait_timeout(vplbm_ctx *c, int enable)
 {
     if (!c) return fail(VPLBM_EINVAL, "context is NULL");
-    if (enable && c->kernel != KERNEL_TMA && !(c->kernel == KERNEL_RESIDENT && c->res_chosen))
+    if (enable && c->kernel != KERNEL_TMA && c->kernel != KERNEL_RESIDENT)
         return fail(VPLBM_EUNSUPPORTED, "neither the TMA-staged nor the resident kernel is selected");
     c->res_mute = enable && c->kernel == KERNEL_RESIDENT;
     c->base.tx_extra = enable && c->kernel == KERNEL_TMA ? 16u : 0u;
@@ -1307,7 +1312,6 @@ vplbm_status vplbm_autotune(vplbm_ctx *c, int steps_per_trial)
     }
     const long long nstep0 = c->nstep;
     const int k0 = c->kernel, bx0 = c->bx, by0 = c->by;
-    const bool chosen0 = c->res_chosen;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     vplbm_status st = VPLBM_OK;
     float best = 1e30f;
@@ -1404,7 +1408,6 @@ vplbm_status vplbm_autotune(vplbm_ctx *c, int steps_per_trial)
     if (e1) cudaEventDestroy(e1);
     cudaFree(save_f);
     cudaFree(save_h);
-    c->res_chosen = chosen0;
     if (best_kernel >= 0) {
         c->kernel = best_kernel;
         c->bx = best_bx;

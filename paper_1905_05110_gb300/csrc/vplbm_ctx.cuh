@@ -48,7 +48,6 @@ struct vplbm_ctx {
     // resident kernel: its tiling, and its mailboxes and rings (allocated by
     // the first resident call, freed by vplbm_destroy)
     bool res_ok = false;
-    bool res_chosen = false;              // by vplbm_set_launch (not the default)
     bool res_mute = false;                // test hook
     vplbm::ResidentPlan res_plan{};
     void *res_ws = nullptr;

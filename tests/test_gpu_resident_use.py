@@ -1,0 +1,73 @@
+"""The resident kernel as a user's program meets it: what the launch queries
+say of a context that runs it by default, after a trial run or on request."""
+import numpy as np
+import pytest
+
+import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _library(gpu_library):
+    return gpu_library
+
+
+def _sim(precision="f32", nx=96, ny=64, **kw):
+    import paper_1905_05110_gb300 as vp
+    p = wl.channel_fixed_disk(nx, ny, diameter=12, center=(30, 31))
+    sim = vp.Simulation(p, precision, history_capacity=64, **kw)
+    sim.init_from_problem()
+    return sim
+
+
+@pytest.mark.parametrize("precision", ["f32", "f64"])
+def test_launch_names_the_kernel_that_runs_and_is_taken_back(precision):
+    sim = _sim(precision)
+    named = sim.launch()
+    assert named[0] == "resident"
+    sim.set_launch("scalar48", 128, 2)
+    assert sim.launch() == ("scalar48", 128, 2)
+    sim.set_launch(*named)
+    assert sim.launch() == named
+    sim.set_launch("scalar48", 128, 2)
+    sim.set_launch("resident")            # keeps the one-step kernel and blocks
+    assert sim.launch() == ("resident", 128, 2)
+    sim.set_launch(*sim.launch())
+    assert sim.launch() == ("resident", 128, 2)
+    one_step = sim.autotune(8)
+    named = sim.launch()
+    assert named == ("resident",) + one_step[1:] and one_step[0] != "resident"
+    other = _sim(precision)
+    other.set_launch(*named)
+    assert other.launch() == named
+    for s in (sim, other):
+        s.step(9)
+    assert np.array_equal(sim.populations(), other.populations())
+    other.close()
+    sim.close()
+
+
+def test_wait_limit_of_a_default_context():
+    import paper_1905_05110_gb300 as vp
+    sim = _sim()
+    vp.vplbm_inject_wait_timeout(sim.ctx, True)
+    sim.step(2)
+    with pytest.raises(vp.VplbmError) as ei:
+        sim.sync()
+    assert ei.value.status == 5
+    vp.vplbm_inject_wait_timeout(sim.ctx, False)
+    sim.init_from_problem()
+    sim.step(8)
+    sim.sync()
+    sim.close()
+
+
+def test_lattice_that_does_not_fit_names_its_kernel():
+    import paper_1905_05110_gb300 as vp
+    sim = vp.Simulation(wl.oscillating_disk(), "f32", history_capacity=64)
+    assert sim.launch() == ("scalar40", 256, 1)
+    with pytest.raises(vp.VplbmError) as ei:
+        sim.set_launch("resident")
+    assert ei.value.status == 6
+    sim.close()
