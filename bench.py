@@ -51,16 +51,16 @@ def dominant_kernel(prec: str, launch, kinds: dict) -> str:
     work = {"two_step": 2 * kinds.get("two_step", 0), "one_step": kinds.get("one_step", 0),
             "tma": kinds.get("tma", 0)}
     top = max(work, key=work.get)
+    if kinds.get("resident", 0):   # of many steps each
+        return f"vp_mrt_resident<{PREC_ID[prec]}, 0>"
     if top == "two_step":
         return f"vp_mrt_step2<{PREC_ID[prec]}, 0, 0>"
     if top == "tma":
         return f"vp_mrt_step_tma<{PREC_ID[prec]}>"
     if launch[0] == "pair":
         return f"vp_mrt_step_pair<{PREC_ID[prec]}, 5, 0>"
-    if launch[0] == "resident":
-        return f"vp_mrt_resident<{PREC_ID[prec]}, 0>"
     # single steps of a two-step choice run the 40-register kernel
-    minb = {"scalar": 4, "scalar48": 5, "scalar40": 6, "fused2": 6, "tma": 6}[launch[0]]
+    minb = {"scalar": 4, "scalar48": 5, "scalar40": 6, "fused2": 6, "tma": 6, "resident": 4 if prec == "f64" else 6}[launch[0]]
     return f"vp_mrt_step<{PREC_ID[prec]}, {minb}, 0, 0>"
 
 
@@ -419,7 +419,7 @@ def run_ours(args, rank, world, local_rank):
             t = time_device(sim, args.steps, stream, torch)
             torch.cuda.synchronize()
             k1 = sim.kernel_launches()
-            samples.append((max_over_ranks(t, world, dev, torch), {k: k1[k] - k0[k] for k in k1}))
+            samples.append((max_over_ranks(t, world, dev, torch), {k: k1[k] - k0.get(k, 0) for k in k1}))
     sim.sync()
     times = sorted(t for t, _ in samples)
     dt, kinds = next(s for s in samples if s[0] == times[REPEATS // 2])
@@ -432,7 +432,7 @@ def run_ours(args, rank, world, local_rank):
     # steps; the one-thread lookahead launches move no lattice bytes)
     peak, peak_kind = measured_peak()
     kname = dominant_kernel(prec, launch, kinds)
-    steps_per_launch = 2 if kname.startswith("vp_mrt_step2<") else 1
+    steps_per_launch = 2 if kname.startswith("vp_mrt_step2<") else args.steps // kinds["resident"] if kinds.get("resident") else 1
     algorithmic = BYTES_PER_NODE[prec] * nodes * args.steps
     achieved = algorithmic / dt / 1e9
     traffic = profiled_traffic(kname, args.workload)

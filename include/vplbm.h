@@ -317,8 +317,8 @@ vplbm_status vplbm_get_body_k(vplbm_ctx *ctx, int k, double q[3], double v[3], l
  *                          about 530 000 nodes (FP32) or 150 000 (FP64)):
  *                          what a context of such a lattice does by default
  *                          and what vplbm_autotune may choose.  One cooperative
- *                          launch runs up to 4096 steps; the launch counts
- *                          count its steps, one VPLBM_LAUNCH_ONE_STEP each.  (block_x,
+ *                          launch runs up to 4096 steps (counted by
+ *                          vplbm_get_resident_launches).  (block_x,
  *                          block_y): the blocks of steps that have to be
  *                          launched one by one (on a stream that is being
  *                          captured, or where a cooperative launch is
@@ -364,8 +364,7 @@ vplbm_status vplbm_autotune(vplbm_ctx *ctx, int steps_per_trial);
  * VPLBM_EUNSUPPORTED unless one of the two is selected. */
 vplbm_status vplbm_inject_wait_timeout(vplbm_ctx *ctx, int enable);
 
-/* Number of step-kernel launches made by vplbm_step since creation (a
- * resident launch counts once for each of its steps)
+/* Number of step-kernel launches made by vplbm_step since creation
  * (vplbm_load restores the count saved in the checkpoint). */
 vplbm_status vplbm_get_launch_count(vplbm_ctx *ctx, long long *launches);
 
@@ -373,8 +372,7 @@ vplbm_status vplbm_get_launch_count(vplbm_ctx *ctx, long long *launches);
  * vplbm_get_kernel_launches):
  *  VPLBM_LAUNCH_ONE_STEP   one time step on a scalar step kernel (any
  *                          register budget, shape, or several bodies) or
- *                          on the node-pair kernel, or one time step of a
- *                          resident launch;
+ *                          on the node-pair kernel;
  *  VPLBM_LAUNCH_TWO_STEP   two time steps on the two-step kernel;
  *  VPLBM_LAUNCH_LOOKAHEAD  the one-thread launch that computes pose n + 1
  *                          of a prescribed path ahead of a run of two-step
@@ -386,10 +384,15 @@ typedef enum {
 } vplbm_launch_kind;
 
 /* counts[k] := launches of kind k that vplbm_step made on this context
- * since its creation (not saved in checkpoints).  Their sum equals the
- * vplbm_get_launch_count increase over the same calls; a caller that reads
- * the counts around a call learns which kernels ran it. */
+ * since its creation (not saved in checkpoints).  Their sum and the resident
+ * launches make the vplbm_get_launch_count increase over the same calls; a
+ * caller that reads the counts around a call learns which kernels ran it. */
 vplbm_status vplbm_get_kernel_launches(vplbm_ctx *ctx, long long counts[VPLBM_LAUNCH_KINDS]);
+
+/* Launches of the resident kernel that vplbm_step made on this context since
+ * its creation, and the time steps they took (a kind of its own, outside the
+ * counts above, whose array keeps its size).  Any pointer may be NULL. */
+vplbm_status vplbm_get_resident_launches(vplbm_ctx *ctx, long long *launches, long long *steps);
 
 /* Write / read a checkpoint: populations (storage precision), body state,
  * step counter and history ring.  vplbm_load requires a context created

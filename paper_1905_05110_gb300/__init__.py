@@ -26,7 +26,7 @@ __all__ = [
     "vplbm_get_populations", "vplbm_get_fields", "vplbm_get_fields_dev", "vplbm_get_history",
     "vplbm_get_body", "vplbm_create_bodies", "vplbm_get_num_bodies", "vplbm_get_history_body",
     "vplbm_get_body_k", "MAX_BODIES", "vplbm_set_launch", "vplbm_get_launch", "vplbm_get_step_launch", "vplbm_autotune",
-    "vplbm_get_launch_count", "vplbm_get_kernel_launches", "vplbm_eval_recip_f32", "LAUNCH_KINDS", "vplbm_save", "vplbm_load", "vplbm_last_error", "vplbm_version",
+    "vplbm_get_launch_count", "vplbm_get_kernel_launches", "vplbm_get_resident_launches", "vplbm_eval_recip_f32", "LAUNCH_KINDS", "vplbm_save", "vplbm_load", "vplbm_last_error", "vplbm_version",
     "vplbm_step_noalloc", "BodyState", "vplbm_inject_wait_timeout", "Batch",
     "vplbm_batch_create", "vplbm_batch_destroy", "vplbm_batch_member", "vplbm_batch_step",
     "vplbm_batch_sync", "vplbm_batch_set_launch", "vplbm_batch_get_launch", "vplbm_batch_autotune",
@@ -136,6 +136,7 @@ _SIGS = {
     "vplbm_get_launch_count": (C.c_int, [_CTX, C.POINTER(C.c_longlong)]),
     "vplbm_get_kernel_launches": (C.c_int, [_CTX, C.POINTER(C.c_longlong)]),
     "vplbm_eval_recip_f32": (C.c_int, [C.c_void_p, C.c_void_p, C.c_longlong, C.c_void_p]),
+    "vplbm_get_resident_launches": (C.c_int, [_CTX, C.POINTER(C.c_longlong), C.POINTER(C.c_longlong)]),
     "vplbm_inject_wait_timeout": (C.c_int, [_CTX, C.c_int]),
     "vplbm_save": (C.c_int, [_CTX, C.c_char_p]),
     "vplbm_load": (C.c_int, [_CTX, C.c_char_p]),
@@ -427,6 +428,13 @@ def vplbm_get_kernel_launches(ctx) -> dict:
     return {k: int(counts[n]) for n, k in enumerate(LAUNCH_KINDS)}
 
 
+def vplbm_get_resident_launches(ctx):
+    """(launches, time steps) of the resident kernel."""
+    n, steps = C.c_longlong(), C.c_longlong()
+    _check(load_library().vplbm_get_resident_launches(ctx, C.byref(n), C.byref(steps)))
+    return int(n.value), int(steps.value)
+
+
 def vplbm_eval_recip_f32(x_ptr: int, y_ptr: int, n: int, stream: int = 0):
     """y[k] := the step kernels' FP32 reciprocal of x[k] (device arrays)."""
     _check(load_library().vplbm_eval_recip_f32(C.c_void_p(x_ptr), C.c_void_p(y_ptr), int(n), C.c_void_p(stream)))
@@ -681,12 +689,15 @@ class Simulation:
 
     @property
     def launches(self) -> int:
-        """Kernel launches made by step() since creation (a resident launch counts once per step)."""
+        """Kernel launches made by step() since creation."""
         return vplbm_get_launch_count(self.ctx)
 
     def kernel_launches(self) -> dict:
-        """Launches made so far by kind: one_step, two_step, lookahead, tma."""
-        return vplbm_get_kernel_launches(self.ctx)
+        """Launches made so far by kind: one_step, two_step, lookahead, tma and, once there are any,
+        resident (each of many steps)."""
+        kinds = vplbm_get_kernel_launches(self.ctx)
+        resident = vplbm_get_resident_launches(self.ctx)[0]
+        return dict(kinds, resident=resident) if resident else kinds
 
     def adjoint(self, nsteps: int, window_start: int, w_cd: float = 1.0, w_cl: float = 0.0,
                 checkpoint_interval: int = 0):

@@ -827,9 +827,9 @@ vplbm_status step_impl(vplbm_ctx *c, long long n)
                 ctx_disable_resident(c);
                 break;
             }
-            // counted by steps, as the launches they stand for
-            c->kcount[VPLBM_LAUNCH_ONE_STEP] += m;
-            c->launches += m;
+            c->res_launches += 1;
+            c->res_steps += m;
+            c->launches += 1;
             n -= m;
         }
     }
@@ -1285,6 +1285,14 @@ vplbm_status vplbm_get_launch_count(vplbm_ctx *c, long long *launches)
 {
     if (!c || !launches) return fail(VPLBM_EINVAL, "NULL argument");
     *launches = c->launches;
+    return VPLBM_OK;
+}
+
+vplbm_status vplbm_get_resident_launches(vplbm_ctx *c, long long *launches, long long *steps)
+{
+    if (!c) return fail(VPLBM_EINVAL, "context is NULL");
+    if (launches) *launches = c->res_launches;
+    if (steps) *steps = c->res_steps;
     return VPLBM_OK;
 }
 

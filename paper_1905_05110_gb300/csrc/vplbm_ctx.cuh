@@ -53,6 +53,7 @@ struct vplbm_ctx {
     void *res_ws = nullptr;
     size_t res_bytes = 0, res_poses = 0, res_parts = 0;
     uint32_t res_tag = 1;                 // tag of the next resident step
+    long long res_launches = 0, res_steps = 0;   // made by vplbm_step
     // device workspace of vplbm_adjoint (checkpoints, segment stores,
     // adjoint fields, accumulators), kept between calls; grown when a call
     // needs more, freed by vplbm_destroy

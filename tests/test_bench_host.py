@@ -150,3 +150,8 @@ def test_reference_band_keeps_the_body_and_walls_the_cut_edges():
     assert q["body"] is not None and 0 <= q["body"]["y"] < 64
     assert abs(q["body"]["y"] - 32) <= 1 and q["body"]["x"] == p["body"]["x"]
     assert bench.row_band(p, p["ny"])["body"]["y"] == p["body"]["y"]
+
+
+def test_dominant_kernel_of_a_resident_region():
+    kinds = {"one_step": 0, "two_step": 0, "lookahead": 0, "tma": 0, "resident": 1}
+    assert bench.dominant_kernel("f32", ("resident", 256, 1), kinds) == "vp_mrt_resident<1, 0>"

@@ -71,3 +71,18 @@ def test_lattice_that_does_not_fit_names_its_kernel():
         sim.set_launch("resident")
     assert ei.value.status == 6
     sim.close()
+
+
+@pytest.mark.parametrize("precision", ["f32", "f64"])
+def test_launch_counts_are_of_launches(precision):
+    import paper_1905_05110_gb300 as vp
+    sim = _sim(precision)
+    sim.step(70)
+    sim.step(1)
+    assert sim.launches == 2 and sim.kernel_launches() == {"one_step": 0, "two_step": 0, "lookahead": 0, "tma": 0, "resident": 2}
+    assert vp.vplbm_get_resident_launches(sim.ctx) == (2, 71)
+    sim.set_launch("scalar48", 128, 2)
+    sim.step(40)
+    assert sim.launches == 42 == sum(sim.kernel_launches().values())
+    sim.sync()
+    sim.close()
