@@ -176,7 +176,7 @@ typedef struct vplbm_ctx vplbm_ctx;
 typedef struct {
     size_t populations;   /* bytes of EACH of the two population buffers */
     size_t body_state;    /* bytes of the body-state pair */
-    size_t partials;      /* bytes of the per-block reduction scratch */
+    size_t partials;      /* bytes of the per-block reduction scratch and the resident kernel's workspace */
     size_t history;       /* bytes of the history ring */
     size_t profiles;      /* bytes of the wall-velocity profiles and the outlet state */
     size_t control;       /* bytes of the ticket / error words */
@@ -326,8 +326,8 @@ vplbm_status vplbm_get_body_k(vplbm_ctx *ctx, int k, double q[3], double v[3], l
  *                          do the blocks that vplbm_get_launch names.  Its
  *                          populations equal the scalar kernel's bit for
  *                          bit; its force sums are added in another order.
- *                          The context keeps a workspace of a few MB for it,
- *                          allocated when a state is set.  A launch takes
+ *                          Its workspace (a few MB) is part of the partials'
+ *                          buffer: stepping allocates nothing.  A launch takes
  *                          every SM: contexts on different streams that
  *                          should overlap choose another kernel (or are the
  *                          members of a batch).

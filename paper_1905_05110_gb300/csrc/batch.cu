@@ -448,10 +448,8 @@ vplbm_status vplbm_batch_create(const vplbm_lattice_desc *lats, const vplbm_body
         delete b;
         return berr(VPLBM_ENOMEM, "host allocation failed");
     }
-    for (int k = 0; k < n && st == VPLBM_OK; ++k) {
-        st = vplbm_create(&lats[k], bodies ? bodies[k] : nullptr, history_capacity, cuda_stream, &b->members[k]);
-        if (st == VPLBM_OK) ctx_disable_resident(b->members[k]);   // members step together, by launches
-    }
+    for (int k = 0; k < n && st == VPLBM_OK; ++k)
+        st = ctx_create_member(&lats[k], bodies ? bodies[k] : nullptr, history_capacity, cuda_stream, &b->members[k]);
     cudaError_t e = cudaSuccess;
     if (st == VPLBM_OK) {
         e = cudaStreamCreateWithFlags(&b->capture, cudaStreamNonBlocking);

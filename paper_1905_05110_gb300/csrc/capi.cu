@@ -154,8 +154,58 @@ long long grid_rows(const vplbm_ctx *c, int bx, int by, int kernel = KERNEL_SCAL
 // have max(nb, 1) slots.
 inline int body_slots(int nb) { return nb > 1 ? nb : 1; }
 
+// Resident kernel: the tiling, and whether this lattice can take it.
+//
+// The lattice has to fit: one tile on every SM but the tail's, of at most as
+// many nodes as its threads hold (resident_k).  Of the tilings that do, the fewest nodes per
+// thread, then the smallest tile, then the shortest edge.  Tiles are at least
+// 8 nodes wide and high (a lattice narrower than 16 is one tile there), since
+// smaller ones exchange more than they update.  Every lattice that fits takes
+// it unless a kernel was asked for: it was faster than the launches at every
+// size measured, by 4.2x at 97 x 70 (2.1 us a step against 8.9), 3.1x at 512 x
+// 256, 1.8x at 900 x 450 and 1.7x at 1230 x 410, where the registers end it.
+bool plan_resident(int nx, int ny, int precision, ResidentPlan *out)
+{
+    constexpr int sms = RES_SMS;
+    int edge_at = 0, smem = 0;
+    long long best = -1;
+    for (int ntx = 1; ntx < sms && (ntx == 1 || nx / ntx >= 8); ++ntx)
+        for (int nty = 1; ntx * nty < sms && (nty == 1 || ny / nty >= 8); ++nty) {
+            const int mw = (nx + ntx - 1) / ntx, mh = (ny + nty - 1) / nty;
+            const int kn = resident_k(precision, mw, mh, &edge_at, &smem);
+            if (kn == 0) continue;
+            const long long cost = ((long long)kn << 40) + ((long long)mw * mh << 20) + mw + mh;
+            if (best < 0 || cost < best) {
+                best = cost;
+                // a tile is at most as many steps behind those that meet the
+                // body as it is tiles away, and these at most 8 behind the tail
+                *out = {ntx, nty, ntx * nty, mw, mh, kn, 8 * (mw + mh), 1, 1, (ntx > nty ? ntx : nty) + 32, edge_at, smem};
+            }
+        }
+    return best >= 0;
+}
+
+// The plan for a lattice and its body, and the workspace it needs (part of the
+// caller's `partials` buffer, so it follows from the descriptors alone).
+bool resident_for(const vplbm_lattice_desc *lat, const vplbm_body_desc *bodies, int nb, ResidentPlan *t, size_t *bytes,
+                  size_t *poses, size_t *parts)
+{
+    if (nb > 1 || !plan_resident(lat->nx, lat->ny, lat->precision, t)) return false;
+    if (nb == 1) {
+        // columns and rows of tiles that the body's node range can meet
+        const long long span = (long long)ceil(2.0 * fmin(bounding_radius(&bodies[0]), 1e6)) + 5;
+        const long long nc = span / (lat->nx / t->ntx) + 2, nr = span / (lat->ny / t->nty) + 2;
+        t->part_slots = (int)((nc < t->ntx ? nc : t->ntx) * (nr < t->nty ? nr : t->nty));
+        if (bodies[0].motion == VPLBM_MOTION_FREE) t->part_copies = 1 + t->part_slots;
+    }
+    *bytes = resident_bytes(*t, lat->precision, poses, parts);
+    return true;
+}
+
+// resident: with the resident kernel's workspace (*res_at: where it starts in
+// the partials; 0 where the lattice does not take that kernel).
 void sizes_for(const vplbm_lattice_desc *lat, const vplbm_body_desc *bodies, int nb, long long cap,
-               vplbm_buffer_sizes *s, long long *ps_out, long long *parts_out)
+               vplbm_buffer_sizes *s, long long *ps_out, long long *parts_out, bool resident = true, size_t *res_at = nullptr)
 {
     const long long n = (long long)lat->nx * lat->ny;
     const long long ps = (long long)round_up((size_t)n, 128);
@@ -188,6 +238,11 @@ void sizes_for(const vplbm_lattice_desc *lat, const vplbm_body_desc *bodies, int
     // one partials region per body; one body: two (one per step of the
     // two-step kernel)
     s->partials = round_up((size_t)(slots > 2 ? slots : 2) * parts * NPART * sizeof(double), ALIGN);
+    ResidentPlan plan;
+    size_t bytes = 0, poses = 0, sums = 0;
+    const bool room = resident && resident_for(lat, bodies, nb, &plan, &bytes, &poses, &sums);
+    if (res_at) *res_at = room ? s->partials : 0;
+    if (room) s->partials += round_up(bytes, ALIGN);
     s->history = round_up((size_t)slots * cap * sizeof(vplbm_record), ALIGN);
     // FP64 profiles, then their FP32 copies: [side][comp][maxlen] each; then
     // the convective outlet state: [parity][3][ny] 8-byte slots
@@ -304,77 +359,25 @@ const char *pair_refusal(const vplbm_ctx *c)
     return nullptr;
 }
 
-// Resident kernel: the tiling, and whether this lattice can take it.
-//
-// The lattice has to fit: one tile on every SM but the tail's, of at most as
-// many nodes as its threads hold (resident_k).  Of the tilings that do, the fewest nodes per
-// thread, then the smallest tile, then the shortest edge.  Tiles are at least
-// 8 nodes wide and high (a lattice narrower than 16 is one tile there), since
-// smaller ones exchange more than they update.  Every lattice that fits takes
-// it unless a kernel was asked for: it was faster than the launches at every
-// size measured, by 4.2x at 97 x 70 (2.1 us a step against 8.9), 3.1x at 512 x
-// 256, 1.8x at 900 x 450 and 1.7x at 1230 x 410, where the registers end it.
-bool plan_resident(int nx, int ny, int precision, int sms, ResidentPlan *out)
-{
-    int edge_at = 0, smem = 0;
-    long long best = -1;
-    for (int ntx = 1; ntx < sms && (ntx == 1 || nx / ntx >= 8); ++ntx)
-        for (int nty = 1; ntx * nty < sms && (nty == 1 || ny / nty >= 8); ++nty) {
-            const int mw = (nx + ntx - 1) / ntx, mh = (ny + nty - 1) / nty;
-            const int kn = resident_k(precision, mw, mh, &edge_at, &smem);
-            if (kn == 0) continue;
-            const long long cost = ((long long)kn << 40) + ((long long)mw * mh << 20) + mw + mh;
-            if (best < 0 || cost < best) {
-                best = cost;
-                // a tile is at most as many steps behind those that meet the
-                // body as it is tiles away, and these at most 8 behind the tail
-                *out = {ntx, nty, ntx * nty, mw, mh, kn, 8 * (mw + mh), 1, 1, (ntx > nty ? ntx : nty) + 32, edge_at, smem};
-            }
-        }
-    return best >= 0;
-}
-
-void setup_resident(vplbm_ctx *c)
+// The resident kernel of a context whose buffers have room for it (at: where
+// its workspace starts in `partials`; 0: none).
+cudaError_t setup_resident(vplbm_ctx *c, const vplbm_lattice_desc *lat, size_t at)
 {
     int sms = 0, coop = 0;
-    c->res_ok = c->nbodies <= 1 && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device) == cudaSuccess &&
+    c->res_ok = at != 0 && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device) == cudaSuccess &&
                 cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, c->device) == cudaSuccess && coop &&
-                plan_resident(c->nx, c->ny, c->precision, sms, &c->res_plan);
-    if (c->res_ok && c->has_body) {
-        // columns and rows of tiles that the body's node range can meet
-        const ResidentPlan &t = c->res_plan;
-        const long long span = (long long)ceil(2.0 * fmin(bounding_radius(&c->body_desc), 1e6)) + 5;
-        const long long nc = span / (c->nx / t.ntx) + 2, nr = span / (c->ny / t.nty) + 2;
-        c->res_plan.part_slots = (int)((nc < t.ntx ? nc : t.ntx) * (nr < t.nty ? nr : t.nty));
-        if (c->body_desc.motion == VPLBM_MOTION_FREE) c->res_plan.part_copies = 1 + c->res_plan.part_slots;
-    }
-    if (c->res_ok) c->res_bytes = resident_bytes(c->res_plan, c->precision, &c->res_poses, &c->res_parts);
-}
-
-// The resident kernel's workspace (a few MB, kept by the context).  Allocated
-// when a state is set, so that stepping allocates nothing.
-cudaError_t ensure_resident(vplbm_ctx *c)
-{
-    if (!c->res_ok || c->kernel != KERNEL_RESIDENT || c->res_ws) return cudaSuccess;
-    const cudaError_t e = cudaMalloc(&c->res_ws, c->res_bytes);
-    if (e != cudaSuccess) {
-        (void)cudaGetLastError();
-        c->res_ws = nullptr;
-        return e;
-    }
-    c->res_tag = 0;
-    return cudaSuccess;
+                resident_for(lat, c->bodies, c->nbodies, &c->res_plan, &c->res_bytes, &c->res_poses, &c->res_parts) &&
+                c->res_plan.tiles < sms;
+    if (!c->res_ok) return cudaSuccess;
+    c->res_ws = reinterpret_cast<char *>(c->partials) + at;
+    return cudaMemsetAsync(c->res_ws, 0, c->res_bytes, c->stream);
 }
 
 // n <= RES_MAX_STEPS steps from the current one in one resident launch
 // (asynchronous); advances the step counter.
 cudaError_t launch_resident_steps(vplbm_ctx *c, int n)
 {
-    {
-        const cudaError_t e = ensure_resident(c);   // a context stepped from the state at rest
-        if (e != cudaSuccess) return e;
-    }
-    if (c->res_tag == 0 || c->res_tag > 0xffffffffu - 2 * RES_MAX_STEPS) {   // new, or the tags are used up
+    if (c->res_tag > 0xffffffffu - 2 * RES_MAX_STEPS) {   // the tags are used up
         const cudaError_t e = cudaMemsetAsync(c->res_ws, 0, c->res_bytes, c->stream);
         if (e != cudaSuccess) return e;
         c->res_tag = 1;
@@ -549,7 +552,7 @@ void fill_dev_body(StepParams &p, const vplbm_lattice_desc *lat, const vplbm_bod
 namespace {
 
 vplbm_status setup(vplbm_ctx *c, const vplbm_lattice_desc *lat, const vplbm_body_desc *bodies, int nb,
-                   long long cap, void *stream)
+                   long long cap, void *stream, size_t res_at)
 {
     const vplbm_body_desc *body = nb > 0 ? &bodies[0] : nullptr;
     c->stream = (cudaStream_t)stream;
@@ -672,7 +675,7 @@ vplbm_status setup(vplbm_ctx *c, const vplbm_lattice_desc *lat, const vplbm_body
     // a lattice that fits the chip's shared memory: the resident kernel, with
     // the above for steps launched one by one
     c->base_kernel = c->kernel;
-    setup_resident(c);
+    CUDA_TRY(setup_resident(c, lat, res_at));
     if (c->res_ok) c->kernel = KERNEL_RESIDENT;
     // populations at rest
     StepParams q = params_for(c, 0);
@@ -683,7 +686,7 @@ vplbm_status setup(vplbm_ctx *c, const vplbm_lattice_desc *lat, const vplbm_body
 }
 
 vplbm_status create_impl(const vplbm_lattice_desc *lat, const vplbm_body_desc *bodies, int nb, long long cap,
-                         void *stream, const vplbm_buffers *user, vplbm_ctx **out)
+                         void *stream, const vplbm_buffers *user, vplbm_ctx **out, bool resident = true)
 {
     if (!out) return fail(VPLBM_EINVAL, "out pointer is NULL");
     *out = nullptr;
@@ -699,7 +702,8 @@ vplbm_status create_impl(const vplbm_lattice_desc *lat, const vplbm_body_desc *b
     if (cap < 1) return fail(VPLBM_EINVAL, "history capacity must be >= 1");
     vplbm_buffer_sizes sz;
     long long ps = 0, parts = 0;
-    sizes_for(lat, bodies, nb, cap, &sz, &ps, &parts);
+    size_t res_at = 0;
+    sizes_for(lat, bodies, nb, cap, &sz, &ps, &parts, resident, &res_at);
 
     vplbm_ctx *c = new (std::nothrow) vplbm_ctx();
     if (!c) return fail(VPLBM_ENOMEM, "host allocation failed");
@@ -740,7 +744,7 @@ vplbm_status create_impl(const vplbm_lattice_desc *lat, const vplbm_body_desc *b
         c->prof = (double *)base; base += sz.profiles;
         c->ctrl = (Control *)base;
     }
-    st = setup(c, lat, bodies, nb, cap, stream);
+    st = setup(c, lat, bodies, nb, cap, stream, res_at);
     if (st != VPLBM_OK) {
         vplbm_destroy(c);
         return st;
@@ -929,6 +933,20 @@ void ctx_disable_resident(vplbm_ctx *c)
 }
 cudaError_t ctx_launch(const vplbm_ctx *c, long long step, cudaStream_t stream) { return launch_one(c, step, stream); }
 vplbm_status ctx_read_error(vplbm_ctx *c) { return read_error(c); }
+vplbm_status ctx_check(const vplbm_lattice_desc *lat, const vplbm_body_desc *body)
+{
+    const vplbm_status st = check_lattice(lat);
+    return st != VPLBM_OK ? st : check_body(body);
+}
+vplbm_status ctx_create_member(const vplbm_lattice_desc *lat, const vplbm_body_desc *body, long long history_capacity,
+                               void *cuda_stream, vplbm_ctx **out)
+{
+    try {
+        return create_impl(lat, body, body ? 1 : 0, history_capacity, cuda_stream, nullptr, out, false);
+    } catch (...) {
+        return fail(VPLBM_ENOMEM, "host allocation failed");
+    }
+}
 }  // namespace vplbm
 
 // ---------------------------------------------------------------- C ABI
@@ -995,7 +1013,6 @@ void vplbm_destroy(vplbm_ctx *c)
     if (c->capture) cudaStreamDestroy(c->capture);
     if (c->owned) cudaFree(c->owned);
     if (c->adj_ws) cudaFree(c->adj_ws);
-    if (c->res_ws) cudaFree(c->res_ws);
     delete c;
 }
 
@@ -1016,7 +1033,6 @@ void *mapped_host(const void *host)
 vplbm_status vplbm_init_equilibrium(vplbm_ctx *c, const double *rho, const double *ux, const double *uy)
 {
     if (!c) return fail(VPLBM_EINVAL, "context is NULL");
-    (void)ensure_resident(c);   // without it the steps are launched one by one
     const size_t n = (size_t)c->nx * c->ny;
     double *tmp = nullptr;
     double *d[3] = {nullptr, nullptr, nullptr};
@@ -1043,7 +1059,6 @@ vplbm_status vplbm_init_equilibrium(vplbm_ctx *c, const double *rho, const doubl
 vplbm_status vplbm_set_populations(vplbm_ctx *c, const double *f)
 {
     if (!c || !f) return fail(VPLBM_EINVAL, "NULL argument");
-    (void)ensure_resident(c);
     try {
         std::vector<char> raw(c->pop_bytes, 0);
         full_to_stored(c, f, raw.data());
@@ -1493,7 +1508,6 @@ vplbm_status vplbm_load(vplbm_ctx *c, const char *path)
              fread(outlet.data(), sizeof(double), outlet.size(), fp) == outlet.size();
         fclose(fp);
         if (!ok) return fail(VPLBM_EIO, "%s is truncated", path);
-        (void)ensure_resident(c);
         const int par = (int)(h.nstep & 1);
         CUDA_TRY(cudaMemcpyAsync(const_cast<void *>(params_for(c, h.nstep).conv_in), outlet.data(),
                                  outlet.size() * sizeof(double), cudaMemcpyHostToDevice, c->stream));

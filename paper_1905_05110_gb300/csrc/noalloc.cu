@@ -27,6 +27,7 @@ namespace vplbm {
 
 // Reports an error message through vplbm_last_error (capi.cu).
 vplbm_status report_error(vplbm_status st, const char *msg);
+vplbm_status ctx_check(const vplbm_lattice_desc *lat, const vplbm_body_desc *body);
 
 namespace {
 
@@ -117,8 +118,7 @@ extern "C" vplbm_status vplbm_step_noalloc(const vplbm_lattice_desc *lat, const 
                                            long long nsteps, void *cuda_stream)
 {
     // host-side checks of the descriptors (no device work, no allocation)
-    vplbm_buffer_sizes sizes;
-    vplbm_status st = vplbm_buffer_sizes_for(lat, body, 1, &sizes);
+    vplbm_status st = ctx_check(lat, body);
     if (st != VPLBM_OK) return st;
     if (!populations_dev || !populations_dev[0] || !populations_dev[1] || !state_dev)
         return report_error(VPLBM_EINVAL, "populations_dev[0..1] and state_dev must be device pointers");

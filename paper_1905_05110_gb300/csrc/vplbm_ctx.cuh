@@ -45,8 +45,7 @@ struct vplbm_ctx {
     bool tma_ok = false;
     CUtensorMap tmap[2];
     int tma_grid = 0;
-    // resident kernel: its tiling, and its mailboxes and rings (allocated by
-    // the first resident call, freed by vplbm_destroy)
+    // resident kernel: its tiling, and its mailboxes and rings (in the partials' buffer)
     bool res_ok = false;
     bool res_mute = false;                // test hook
     vplbm::ResidentPlan res_plan{};
@@ -65,7 +64,12 @@ namespace vplbm {
 // Shared runtime helpers (capi.cu).
 StepParams ctx_params(const vplbm_ctx *c, long long step);        // parameters of step `step`
 inline int step_kernel(const vplbm_ctx *c) { return c->kernel == KERNEL_RESIDENT ? c->base_kernel : c->kernel; }
-void ctx_disable_resident(vplbm_ctx *c);                          // a batch's members step by launches
+void ctx_disable_resident(vplbm_ctx *c);                          // after a refused launch
+vplbm_status ctx_check(const vplbm_lattice_desc *lat, const vplbm_body_desc *body);   // the descriptors' values
+// A batch's member: library-allocated memory, no resident kernel (members step
+// together, by launches).
+vplbm_status ctx_create_member(const vplbm_lattice_desc *lat, const vplbm_body_desc *body, long long history_capacity,
+                               void *cuda_stream, vplbm_ctx **out);
 cudaError_t ctx_launch(const vplbm_ctx *c, long long step, cudaStream_t stream);
 vplbm_status ctx_read_error(vplbm_ctx *c);                          // latched device errors (syncs)
 vplbm_status report_error(vplbm_status st, const char *msg);

@@ -306,6 +306,7 @@ cudaError_t launch_sweep(int precision, bool disk, bool psmem, const SweepLaunch
 // Resident kernel (step_resident.cu): many steps of a small lattice in one
 // cooperative launch of tiles + 1 blocks, the populations in shared memory.
 constexpr int RES_PART_RING = 16;      // steps of partial sums in flight (a tile is at most 8 steps ahead of the tail)
+constexpr int RES_SMS = 152;           // SMs the tiling is made for; a device with fewer takes the lattice's launches
 constexpr int RES_MAX_STEPS = 4096;    // steps of one launch at most (a few milliseconds)
 struct ResidentPlan {
     int ntx, nty, tiles;   // tile columns and rows (tiles of nx / ntx x ny / nty nodes, rounded up or down)

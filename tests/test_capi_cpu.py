@@ -82,3 +82,16 @@ def test_invalid_body_rejected_on_host(lib):
         vp.vplbm_buffer_sizes_for(vp.lattice_desc(p, "f32"), vp.body_desc(b), 10)
     with pytest.raises(vp.VplbmError):
         vp.vplbm_buffer_sizes_for(vp.lattice_desc(p, "f32"), vp.body_desc(p["body"]), 0)
+
+
+def test_buffer_sizes_hold_the_resident_workspace(lib):
+    # tagged words {value, tag}: two parities of four values for every place around each tile, a value of FP64 in two words
+    p = wl.channel_fixed_disk(256, 128, diameter=16, center=(80, 65))
+    size = {prec: vp.vplbm_buffer_sizes_for(vp.lattice_desc(p, prec), vp.body_desc(p["body"]), 10).partials
+            for prec in ("f64", "f32", "f16")}
+    edge = 2 * 4 * 2 * (256 + 128) * 8
+    assert size["f32"] > size["f16"] + edge and size["f64"] > size["f16"] + 2 * edge
+    big = wl.oscillating_disk()   # does not fit the kernel
+    sizes = [vp.vplbm_buffer_sizes_for(vp.lattice_desc(big, prec), vp.body_desc(big["body"]), 10).partials
+             for prec in ("f32", "f16")]
+    assert sizes[0] == sizes[1]

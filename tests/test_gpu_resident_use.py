@@ -86,3 +86,29 @@ def test_launch_counts_are_of_launches(precision):
     assert sim.launches == 42 == sum(sim.kernel_launches().values())
     sim.sync()
     sim.close()
+
+
+@pytest.mark.parametrize("precision", ["f32", "f64"])
+def test_no_device_memory_beside_the_callers_buffers(precision):
+    """A free body's workspace is of some MB; a context on the caller's buffers takes it from these."""
+    import torch
+    import paper_1905_05110_gb300 as vp
+    nx, ny = (700, 400) if precision == "f32" else (400, 240)
+    r = ny / 3.0
+    body = {"radius": r, "x": nx * 0.5, "y": ny * 0.5, "motion": "free", "mass": 4 * r * r, "inertia": r ** 4, "dof_mask": 7,
+            "u_ref": 0.05, "d_ref": 2 * r}
+    sim = vp.Simulation(wl.mixed_bc_box(nx, ny, seed=2, body=body), precision, history_capacity=64)
+    assert sim.launch()[0] == "resident"
+    f = sim.populations()
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    for state in ("rest", "equilibrium", "populations"):
+        if state == "equilibrium":
+            sim.init_equilibrium()
+        elif state == "populations":
+            sim.set_populations(f)
+        sim.step(20)
+        sim.sync()
+    assert torch.cuda.mem_get_info()[0] == free
+    assert vp.vplbm_get_resident_launches(sim.ctx) == (3, 60)
+    sim.close()
