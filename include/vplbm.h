@@ -321,8 +321,9 @@ vplbm_status vplbm_get_body_k(vplbm_ctx *ctx, int k, double q[3], double v[3], l
  *                          vplbm_get_resident_launches).  (block_x,
  *                          block_y): the blocks of steps that have to be
  *                          launched one by one (on a stream that is being
- *                          captured, or where a cooperative launch is
- *                          refused); 0 x 0 keeps the current ones, and so
+ *                          captured, or where the device cannot hold the
+ *                          cooperative launch, which every call tries
+ *                          again); 0 x 0 keeps the current ones, and so
  *                          do the blocks that vplbm_get_launch names.  Its
  *                          populations equal the scalar kernel's bit for
  *                          bit; its force sums are added in another order.
@@ -361,6 +362,8 @@ vplbm_status vplbm_autotune(vplbm_ctx *ctx, int steps_per_trial);
  * its tensor copies deliver, so the wait gives up after about one second,
  * the block leaves once its copies have landed, and the next vplbm_sync
  * returns VPLBM_ETIMEOUT; the context stays usable.  Disable to resume.
+ * enable 2, resident kernel: no wait runs out, but its launches are refused
+ * as on a device with too few free SMs (the steps are launched one by one).
  * VPLBM_EUNSUPPORTED unless one of the two is selected. */
 vplbm_status vplbm_inject_wait_timeout(vplbm_ctx *ctx, int enable);
 

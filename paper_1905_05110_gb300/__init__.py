@@ -407,8 +407,8 @@ def vplbm_autotune(ctx, steps_per_trial: int = 20):
     _check(load_library().vplbm_autotune(ctx, int(steps_per_trial)))
 
 
-def vplbm_inject_wait_timeout(ctx, enable: bool):
-    _check(load_library().vplbm_inject_wait_timeout(ctx, int(bool(enable))))
+def vplbm_inject_wait_timeout(ctx, enable: int):
+    _check(load_library().vplbm_inject_wait_timeout(ctx, 2 if enable == 2 else int(bool(enable))))
 
 
 def vplbm_get_launch_count(ctx) -> int:

@@ -377,6 +377,7 @@ cudaError_t setup_resident(vplbm_ctx *c, const vplbm_lattice_desc *lat, size_t a
 // (asynchronous); advances the step counter.
 cudaError_t launch_resident_steps(vplbm_ctx *c, int n)
 {
+    if (c->res_refuse) return cudaErrorCooperativeLaunchTooLarge;
     if (c->res_tag > 0xffffffffu - 2 * RES_MAX_STEPS) {   // the tags are used up
         const cudaError_t e = cudaMemsetAsync(c->res_ws, 0, c->res_bytes, c->stream);
         if (e != cudaSuccess) return e;
@@ -403,6 +404,14 @@ cudaError_t launch_resident_steps(vplbm_ctx *c, int n)
     c->res_tag += (uint32_t)n + 1;
     c->nstep += n;
     return cudaSuccess;
+}
+
+// Whether a resident launch failed because the device cannot hold it now (the
+// process has fewer SMs or less memory than the device): the steps are then
+// launched one by one.  Any other error is the call's.
+bool resident_refused(cudaError_t e)
+{
+    return e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorLaunchOutOfResources || e == cudaErrorMemoryAllocation;
 }
 
 // Steps of one captured graph, launches per graph.
@@ -826,10 +835,11 @@ vplbm_status step_impl(vplbm_ctx *c, long long n)
         }
         while (n > 0 && cap == cudaStreamCaptureStatusNone) {
             const int m = (int)(n < RES_MAX_STEPS ? n : RES_MAX_STEPS);
-            if (launch_resident_steps(c, m) != cudaSuccess) {   // no memory, or too few SMs left to this process
+            const cudaError_t e = launch_resident_steps(c, m);
+            if (e != cudaSuccess) {
                 (void)cudaGetLastError();
-                ctx_disable_resident(c);
-                break;
+                if (!resident_refused(e)) return fail(VPLBM_ECUDA, "resident launch failed: %s", cudaGetErrorString(e));
+                break;   // the rest of this call; the next one tries again
             }
             c->res_launches += 1;
             c->res_steps += m;
@@ -926,11 +936,6 @@ struct CkptHeader {
 
 namespace vplbm {
 StepParams ctx_params(const vplbm_ctx *c, long long step) { return params_for(c, step); }
-void ctx_disable_resident(vplbm_ctx *c)
-{
-    c->res_ok = false;
-    c->kernel = step_kernel(c);
-}
 cudaError_t ctx_launch(const vplbm_ctx *c, long long step, cudaStream_t stream) { return launch_one(c, step, stream); }
 vplbm_status ctx_read_error(vplbm_ctx *c) { return read_error(c); }
 vplbm_status ctx_check(const vplbm_lattice_desc *lat, const vplbm_body_desc *body)
@@ -1290,7 +1295,8 @@ vplbm_status vplbm_inject_wait_timeout(vplbm_ctx *c, int enable)
     if (!c) return fail(VPLBM_EINVAL, "context is NULL");
     if (enable && c->kernel != KERNEL_TMA && c->kernel != KERNEL_RESIDENT)
         return fail(VPLBM_EUNSUPPORTED, "neither the TMA-staged nor the resident kernel is selected");
-    c->res_mute = enable && c->kernel == KERNEL_RESIDENT;
+    c->res_mute = enable && enable != 2 && c->kernel == KERNEL_RESIDENT;
+    c->res_refuse = enable == 2 && c->kernel == KERNEL_RESIDENT;
     c->base.tx_extra = enable && c->kernel == KERNEL_TMA ? 16u : 0u;
     c->graph_kernel = -1;   // recapture graphs with the new parameters
     return VPLBM_OK;
@@ -1401,9 +1407,8 @@ vplbm_status vplbm_autotune(vplbm_ctx *c, int steps_per_trial)
                     if (launch_resident_steps(c, m) != cudaSuccess) break;
                     s += m;
                 }
-                if (res && c->nstep != nstep0 + steps_per_trial) {   // cannot be launched here
+                if (res && c->nstep != nstep0 + steps_per_trial) {   // cannot be launched now
                     (void)cudaGetLastError();
-                    ctx_disable_resident(c);
                     break;
                 }
                 for (int s = 0; !two && !res && s < steps_per_trial && st == VPLBM_OK; ++s) {

@@ -47,7 +47,7 @@ struct vplbm_ctx {
     int tma_grid = 0;
     // resident kernel: its tiling, and its mailboxes and rings (in the partials' buffer)
     bool res_ok = false;
-    bool res_mute = false;                // test hook
+    bool res_mute = false, res_refuse = false;   // test hooks
     vplbm::ResidentPlan res_plan{};
     void *res_ws = nullptr;
     size_t res_bytes = 0, res_poses = 0, res_parts = 0;
@@ -64,7 +64,6 @@ namespace vplbm {
 // Shared runtime helpers (capi.cu).
 StepParams ctx_params(const vplbm_ctx *c, long long step);        // parameters of step `step`
 inline int step_kernel(const vplbm_ctx *c) { return c->kernel == KERNEL_RESIDENT ? c->base_kernel : c->kernel; }
-void ctx_disable_resident(vplbm_ctx *c);                          // after a refused launch
 vplbm_status ctx_check(const vplbm_lattice_desc *lat, const vplbm_body_desc *body);   // the descriptors' values
 // A batch's member: library-allocated memory, no resident kernel (members step
 // together, by launches).

@@ -112,3 +112,22 @@ def test_no_device_memory_beside_the_callers_buffers(precision):
     assert torch.cuda.mem_get_info()[0] == free
     assert vp.vplbm_get_resident_launches(sim.ctx) == (3, 60)
     sim.close()
+
+
+def test_a_refused_launch_is_not_the_end_of_the_kernel():
+    import paper_1905_05110_gb300 as vp
+    a, b = _sim(), _sim()
+    a.set_launch("resident", 128, 2)
+    a.step(5)
+    vp.vplbm_inject_wait_timeout(a.ctx, 2)
+    a.step(40)      # launched one by one
+    assert a.kernel_launches() == {"one_step": 40, "two_step": 0, "lookahead": 0, "tma": 0, "resident": 1}
+    assert a.autotune(4)[0] != "resident" and a.launch()[0] != "resident"   # measured what can be launched
+    a.set_launch("resident")
+    vp.vplbm_inject_wait_timeout(a.ctx, 0)
+    a.step(7)
+    assert a.kernel_launches()["resident"] == 2
+    b.step(52)
+    assert np.array_equal(a.populations(), b.populations())
+    a.close()
+    b.close()
