@@ -317,7 +317,7 @@ vplbm_status vplbm_get_body_k(vplbm_ctx *ctx, int k, double q[3], double v[3], l
  *                          about 530 000 nodes (FP32) or 150 000 (FP64)):
  *                          what a context of such a lattice does by default
  *                          and what vplbm_autotune may choose.  One cooperative
- *                          launch runs up to 4096 steps (counted by
+ *                          launch runs up to 1024 steps (counted by
  *                          vplbm_get_resident_launches).  (block_x,
  *                          block_y): the blocks of steps that have to be
  *                          launched one by one (on a stream that is being
@@ -329,9 +329,13 @@ vplbm_status vplbm_get_body_k(vplbm_ctx *ctx, int k, double q[3], double v[3], l
  *                          bit; its force sums are added in another order.
  *                          Its workspace (a few MB) is part of the partials'
  *                          buffer: stepping allocates nothing.  A launch takes
- *                          every SM: contexts on different streams that
- *                          should overlap choose another kernel (or are the
- *                          members of a batch).
+ *                          every SM for 2 to 10 ms, so contexts on streams
+ *                          of their own run one after another: while the
+ *                          process has contexts that fit this kernel on more
+ *                          than 3 streams of the device (FP64 storage: 2),
+ *                          they step by single launches, which overlap,
+ *                          unless vplbm_set_launch asked for the resident
+ *                          kernel.
  * Nodes on the lattice edges and near the body always take the same code.
  * The results of different kernels agree to the rounding of the storage
  * precision. */

@@ -6,6 +6,8 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <map>
+#include <mutex>
 #include <new>
 #include <string>
 #include <vector>
@@ -373,6 +375,56 @@ cudaError_t setup_resident(vplbm_ctx *c, const vplbm_lattice_desc *lat, size_t a
     return cudaMemsetAsync(c->res_ws, 0, c->res_bytes, c->stream);
 }
 
+// Streams with live contexts that fit the resident kernel, per device.  Its
+// launch takes every SM, so such contexts on streams of their own run one
+// after another, where single launches overlap; and the more of them, the
+// more that costs.  us a step of all of n contexts, launches / resident:
+//   FP32  97 x 70 fixed disk  n = 3: 9.5 / 6.3   4: 9.8 / 8.2    6: 10.1 / 12.6   16: 17.2 / 33.4
+//         512 x 256 free           3: 16.7 / 14.9   4: 17.2 / 20.0
+//         700 x 400 fixed          3: 14.4 / 14.1   4: 16.6 / 18.7
+//   FP64  256 x 128 fixed     n = 2: 16.3 / 12.9   3: 17.2 / 19.5   16: 39.8 / 103
+//         512 x 256 fixed          2: 19.5 / 19.6   3: 21.8 / 29.5
+// So with more than 3 (FP64: 2) of these streams a context steps by launches,
+// unless it was asked to do otherwise by vplbm_set_launch.
+struct StreamUse {
+    std::mutex m;
+    std::map<int, std::map<cudaStream_t, int>> contexts;   // [device][stream]
+};
+StreamUse &stream_use()
+{
+    static StreamUse *u = new StreamUse;   // outlives every context
+    return *u;
+}
+
+bool enter_stream(const vplbm_ctx *c)
+{
+    try {
+        StreamUse &u = stream_use();
+        const std::lock_guard<std::mutex> lock(u.m);
+        ++u.contexts[c->device][c->stream];
+        return true;
+    } catch (...) {
+        return false;
+    }
+}
+
+void leave_stream(const vplbm_ctx *c)
+{
+    StreamUse &u = stream_use();
+    const std::lock_guard<std::mutex> lock(u.m);
+    auto &streams = u.contexts[c->device];
+    if (--streams[c->stream] == 0) streams.erase(c->stream);
+}
+
+// Whether the context's next steps run on the resident kernel.
+bool resident_now(const vplbm_ctx *c)
+{
+    if (c->kernel != KERNEL_RESIDENT || c->res_asked) return c->kernel == KERNEL_RESIDENT;
+    StreamUse &u = stream_use();
+    const std::lock_guard<std::mutex> lock(u.m);
+    return (int)u.contexts[c->device].size() <= (c->precision == VPLBM_F64 ? 2 : 3);
+}
+
 // n <= RES_MAX_STEPS steps from the current one in one resident launch
 // (asynchronous); advances the step counter.
 cudaError_t launch_resident_steps(vplbm_ctx *c, int n)
@@ -685,6 +737,7 @@ vplbm_status setup(vplbm_ctx *c, const vplbm_lattice_desc *lat, const vplbm_body
     // the above for steps launched one by one
     c->base_kernel = c->kernel;
     CUDA_TRY(setup_resident(c, lat, res_at));
+    if (c->res_ok) c->res_ok = c->res_entered = enter_stream(c);
     if (c->res_ok) c->kernel = KERNEL_RESIDENT;
     // populations at rest
     StepParams q = params_for(c, 0);
@@ -825,7 +878,7 @@ vplbm_status step_pairs(vplbm_ctx *c, long long pairs)
 // end (and one at its start, from an odd step, before a graph).
 vplbm_status step_impl(vplbm_ctx *c, long long n)
 {
-    if (c->kernel == KERNEL_RESIDENT && n > 0) {
+    if (n > 0 && resident_now(c)) {
         // a captured launch would replay its tags: steps of a stream that is
         // being captured are launched one by one
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -1014,6 +1067,7 @@ void vplbm_destroy(vplbm_ctx *c)
 {
     if (!c) return;
     if (c->stream || c->owned) cudaStreamSynchronize(c->stream);
+    if (c->res_entered) leave_stream(c);
     if (c->graph) cudaGraphExecDestroy(c->graph);
     if (c->capture) cudaStreamDestroy(c->capture);
     if (c->owned) cudaFree(c->owned);
@@ -1229,6 +1283,7 @@ vplbm_status vplbm_set_launch(vplbm_ctx *c, int kernel, int bx, int by)
             c->base_kernel = k0;
         }
         c->kernel = KERNEL_RESIDENT;
+        c->res_asked = true;
         return VPLBM_OK;
     }
     if (kernel == KERNEL_FUSED2) {
@@ -1277,7 +1332,7 @@ vplbm_status vplbm_set_launch(vplbm_ctx *c, int kernel, int bx, int by)
 vplbm_status vplbm_get_launch(vplbm_ctx *c, int *kernel, int *bx, int *by)
 {
     if (!c) return fail(VPLBM_EINVAL, "context is NULL");
-    if (kernel) *kernel = c->kernel;
+    if (kernel) *kernel = resident_now(c) ? (int)KERNEL_RESIDENT : step_kernel(c);
     if (bx) *bx = c->bx;
     if (by) *by = c->by;
     return VPLBM_OK;
@@ -1341,6 +1396,7 @@ vplbm_status vplbm_autotune(vplbm_ctx *c, int steps_per_trial)
     }
     const long long nstep0 = c->nstep;
     const int k0 = c->kernel, bx0 = c->bx, by0 = c->by;
+    const bool asked0 = c->res_asked;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     vplbm_status st = VPLBM_OK;
     float best = 1e30f;
@@ -1436,6 +1492,7 @@ vplbm_status vplbm_autotune(vplbm_ctx *c, int steps_per_trial)
     if (e1) cudaEventDestroy(e1);
     cudaFree(save_f);
     cudaFree(save_h);
+    c->res_asked = asked0;
     if (best_kernel >= 0) {
         c->kernel = best_kernel;
         c->bx = best_bx;

@@ -47,6 +47,8 @@ struct vplbm_ctx {
     int tma_grid = 0;
     // resident kernel: its tiling, and its mailboxes and rings (in the partials' buffer)
     bool res_ok = false;
+    bool res_asked = false;               // for by vplbm_set_launch (not the default or autotune's choice)
+    bool res_entered = false;             // counted among the streams in use
     bool res_mute = false, res_refuse = false;   // test hooks
     vplbm::ResidentPlan res_plan{};
     void *res_ws = nullptr;

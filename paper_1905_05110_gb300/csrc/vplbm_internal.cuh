@@ -307,7 +307,10 @@ cudaError_t launch_sweep(int precision, bool disk, bool psmem, const SweepLaunch
 // cooperative launch of tiles + 1 blocks, the populations in shared memory.
 constexpr int RES_PART_RING = 16;      // steps of partial sums in flight (a tile is at most 8 steps ahead of the tail)
 constexpr int RES_SMS = 152;           // SMs the tiling is made for; a device with fewer takes the lattice's launches
-constexpr int RES_MAX_STEPS = 4096;    // steps of one launch at most (a few milliseconds)
+// Steps of one launch at most: 2.2 ms (97 x 70, FP32) to 10 ms (512 x 256,
+// FP64), for which other streams' work waits.  97 x 70, us a step in launches
+// of 256, 512, 1024, 4096 steps: 2.161, 2.138, 2.128, 2.120.
+constexpr int RES_MAX_STEPS = 1024;
 struct ResidentPlan {
     int ntx, nty, tiles;   // tile columns and rows (tiles of nx / ntx x ny / nty nodes, rounded up or down)
     int mw, mh;            // largest tile width and height

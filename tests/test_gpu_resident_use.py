@@ -136,3 +136,36 @@ def test_a_refused_launch_is_not_the_end_of_the_kernel():
     assert np.array_equal(a.populations(), b.populations())
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("precision,limit", [("f32", 3), ("f64", 2)])
+def test_contexts_on_many_streams_step_by_launches(precision, limit):
+    """Resident launches of different streams cannot overlap: beyond the limit the contexts' single launches do."""
+    import torch
+    streams = [torch.cuda.Stream() for _ in range(limit)]
+    sims = [_sim(precision, stream=s) for s in streams]
+    same = _sim(precision, stream=streams[0])           # on a stream in use already
+    assert all(s.launch()[0] == "resident" for s in sims + [same])
+    asked = _sim(precision, stream=torch.cuda.Stream())
+    crowd = sims + [same]
+    assert all(s.launch()[0] != "resident" for s in crowd + [asked])
+    asked.set_launch("resident")
+    assert asked.launch()[0] == "resident"
+    for s in crowd + [asked]:
+        s.step(40)
+    for s in crowd + [asked]:
+        s.sync()
+    assert all(s.kernel_launches() == {"one_step": 40, "two_step": 0, "lookahead": 0, "tma": 0} for s in crowd)
+    assert asked.kernel_launches()["resident"] == 1
+    asked.close()
+    assert all(s.launch()[0] == "resident" for s in crowd)
+    for s in crowd:
+        s.step(9)
+        s.sync()
+        assert s.kernel_launches()["resident"] == 1
+        assert np.array_equal(s.populations(), crowd[0].populations())
+    ref = _sim(precision, stream=streams[0])
+    ref.step(49)
+    assert np.array_equal(ref.populations(), crowd[0].populations())
+    for s in crowd + [ref]:
+        s.close()
