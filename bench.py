@@ -88,6 +88,20 @@ def bench_config(p: dict, prec: str, world: int) -> dict:
                   if pop_mb > 129 else f"not flushed: populations {pop_mb:.0f} MB per step fit the 129 MB L2"}
 
 
+def json_line(line: dict) -> str:
+    """The report as JSON, where a value that is not finite (no oscillation to
+    measure a frequency of) is null: NaN is not JSON."""
+    def plain(v):
+        if isinstance(v, dict):
+            return {k: plain(x) for k, x in v.items()}
+        if isinstance(v, (list, tuple)):
+            return [plain(x) for x in v]
+        if isinstance(v, (float, np.floating)):
+            return float(v) if np.isfinite(v) else None
+        return v
+    return json.dumps(plain(line), allow_nan=False)
+
+
 def dist_env():
     return int(os.environ.get("RANK", "0")), int(os.environ.get("WORLD_SIZE", "1")), \
         int(os.environ.get("LOCAL_RANK", "0"))
@@ -374,7 +388,7 @@ def run_reference(args, rank, world):
             "impl": "reference",
             "cpu_baseline": {"value": value, "unit": UNIT, "cores": cores, "kind": "oracle", "sample": desc},
             "e2e": {"value": value, "unit": UNIT, "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0}}
-    print(json.dumps(line), flush=True)
+    print(json_line(line), flush=True)
 
 
 def run_ours(args, rank, world, local_rank):
@@ -506,7 +520,7 @@ def run_ours(args, rank, world, local_rank):
                 "config": bench_config(p, prec, world), "launch": list(launch), "repeats": repeats,
                 "roofline": roofline, "cpu_baseline": base, "e2e": e2e,
                 "gpu_launches": launches, "clocks": clock, "compare": compare}
-        print(json.dumps(line), flush=True)
+        print(json_line(line), flush=True)
     sim.close()
 
 

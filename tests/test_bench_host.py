@@ -155,3 +155,13 @@ def test_reference_band_keeps_the_body_and_walls_the_cut_edges():
 def test_dominant_kernel_of_a_resident_region():
     kinds = {"one_step": 0, "two_step": 0, "lookahead": 0, "tma": 0, "resident": 1}
     assert bench.dominant_kernel("f32", ("resident", 256, 1), kinds) == "vp_mrt_resident<1, 0>"
+
+
+def test_report_line_is_json_whatever_the_values():
+    import json
+
+    def no_constant(name):
+        raise ValueError(name)
+    line = {"value": np.float64(2.5), "n": 3, "none": None, "ok": True, "members": [{"omega": float("nan"), "k": np.inf}, (1.0, -np.inf)]}
+    got = json.loads(bench.json_line(line), parse_constant=no_constant)
+    assert got == {"value": 2.5, "n": 3, "none": None, "ok": True, "members": [{"omega": None, "k": None}, [1.0, None]]}
