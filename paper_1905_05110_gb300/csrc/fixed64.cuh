@@ -53,6 +53,15 @@ struct FxFactor {
     int hi, lo;
 };
 
+// The factor of a double in (0, 1/2) known at compile time.
+constexpr FxFactor fx_const(double r)
+{
+    const long long v = (long long)(r * 0x1p64);   // exact: 53 bits
+    const int lo = (int)(uint32_t)(uint64_t)v;
+    return {(int)((v - (long long)lo) >> 32), lo};
+}
+constexpr FxFactor FX_W0 = fx_const(4.0 / 9.0), FX_W1 = fx_const(1.0 / 9.0), FX_W2 = fx_const(1.0 / 36.0);
+
 // Host-folded constants of the fixed-point update (uniform over a run).
 struct FixedConsts {
     int ok;                     // the run's rho0, g and factors are in range
@@ -64,13 +73,12 @@ struct FixedConsts {
     // stress, 1/6, and pen_k / 8 (pen_k = 1 / (eta + 1/2) tends to 2)
     FxFactor h1, h2, h4, h6, h7, h8, sixth, k8;
     long long gvx, gvy;         // g 2^60, for the velocity j / rho + g / 2
-    // g / 16 for the force rho g: two digits (2^-64) would put it off by up to
-    // 4e-19, every step with the same sign
+    // g / 48 for the force rho g / 6 that a population takes, to 2^-96 (from g
+    // 2^60 it would be off by up to 4e-19, every step with the same sign)
     FxFactor gx, gy;
     int gx3, gy3;               // its third digits (2^-96)
     int forced;                 // g is not zero
     long long rho0;             // in units of 2^(E - 59)
-    FxFactor w0, w1, w2;        // the weights
 };
 
 // ok is cleared where the digits do not hold r.
@@ -87,7 +95,7 @@ inline FxFactor fx_factor(double r, int &ok)
     return f;
 }
 
-// g / 16 and its third digit.  other: the other component.  A force of a few
+// g / 48 and its third digit.  other: the other component.  A force of a few
 // units or less is not rounded without a bias (a uniform density rounds it the
 // same way everywhere): below 2^-40 the run takes the FP64 instructions, but
 // for a component that is only the other's rounding (a direction at right
@@ -95,7 +103,7 @@ inline FxFactor fx_factor(double r, int &ok)
 inline FxFactor fx_accel(double g, double other, int &third, int &ok)
 {
     if (g != 0.0 && fabs(g) < 0x1p-40 && !(fabs(g) <= 0x1p-50 * fabs(other))) ok = 0;
-    const double r = g / 16.0, rest = ldexp(r, 64) - rint(ldexp(r, 64));   // both exact, or below 2^-96
+    const double r = g / 48.0, rest = ldexp(r, 64) - rint(ldexp(r, 64));
     third = (int)fmin(rint(ldexp(rest, 32)), 2147483647.0);
     return fx_factor(r, ok);
 }
@@ -127,7 +135,6 @@ inline void fold_fixed(FixedConsts &k, const double *s, double rho0, double gx, 
     k.gy = fx_accel(gy, gx, k.gy3, ok);
     k.forced = gx != 0.0 || gy != 0.0;
     k.rho0 = llrint(ldexp(rho0, 59 - e));
-    k.w0 = fx_factor(4.0 / 9.0, ok); k.w1 = fx_factor(1.0 / 9.0, ok); k.w2 = fx_factor(1.0 / 36.0, ok);
     k.ok = ok;
 }
 
@@ -263,7 +270,7 @@ VPLBM_FX long long fx_recip(long long rho)
     const float inv = 1.0f / rf;
 #endif
     const uint32_t r0 = (uint32_t)(inv * 1152921504606846976.0f);   // 2^60 / (rho 2^-28) = 2^88 / rho
-    // 2^88 - rho r0 in units of 2^16: |d| 2^72 < 2^52
+    // d = (2^88 - rho r0) / 2^16, the residual in units of 2^-72: |d| < 2^52
     const uint64_t pl = (uint64_t)rl * r0;
     const uint64_t ph = (uint64_t)rh * r0 + (pl >> 32);
     long long d = -(long long)((ph << 16) | ((uint32_t)pl >> 16));
@@ -277,19 +284,19 @@ VPLBM_FX long long fx_recip(long long rho)
 // acceleration) does differently, a function of its own on the device: few
 // nodes take it, and inlined it costs the others registers.  In: the moments
 // (v: velocity times 2^61) and the solid velocity us; out: the increments
-// along the rows of M, G / 6, what an axis population takes beside that under
-// a uniform acceleration (r), and a 2^60 of the penalization.  False if the
-// slip is out of range.
+// along the rows of M and G / 6, and a 2^60 of the penalization.  False if
+// the slip is out of range.
 struct FxForced {
     long long rho, jx, jy, vx, vy, usx, usy, f0, sa, sd, qx, qy, pxx, pxy;   // in
-    long long de, dep, dqx, dqy, dp, dr, gx6, gy6, rx, ry, ax, ay;           // out
+    long long de, dep, dqx, dqy, dp, dr, gx6, gy6, ax, ay;                   // out
 };
 
 // G: the lattice may be under a uniform acceleration.
 template <bool G>
 VPLBM_FX bool fx_forced_here(const FixedConsts &k, bool chi, FxForced &w)
 {
-    const long long wx = w.vx + k.gvx, wy = w.vy + k.gvy;   // v = j / rho + g / 2
+    const long long gx = G ? k.gvx : 0, gy = G ? k.gvy : 0;
+    const long long wx = w.vx + gx, wy = w.vy + gy;   // v = j / rho + g / 2
     long long ax = 0, ay = 0;                               // a 2^60
     if (chi) {
         const long long lx = w.usx - wx, ly = w.usy - wy;
@@ -300,27 +307,19 @@ VPLBM_FX bool fx_forced_here(const FixedConsts &k, bool chi, FxForced &w)
     }
     const FxFactor ux = fx_split(wx + ax), uy = fx_split(wy + ay);   // u = v + a / 2
     const long long r8 = (long long)((uint64_t)w.rho << 3);
-    long long Gx, Gy;   // rho (a + g)
+    const long long Gx = fx_mul(r8, fx_split(2 * (ax + gx))), Gy = fx_mul(r8, fx_split(2 * (ay + gy)));
     if (!G || !k.forced) {
-        Gx = fx_mul(r8, fx_split(2 * ax));
-        Gy = fx_mul(r8, fx_split(2 * ay));
         w.gx6 = fx_mul(Gx, k.sixth);
         w.gy6 = fx_mul(Gy, k.sixth);
     } else {
-        // half of it is rounded, and what the four diagonal populations do not
-        // take of a sixth each goes to the other two: the node gains Gx, while
-        // six roundings of Gx / 6 favour the sign of g by half a unit
-        long long hx = fx_mul3(r8, k.gx, k.gx3), hy = fx_mul3(r8, k.gy, k.gy3);
+        // rho g / 6 in one rounding: that of a sixth of Gx, a whole number,
+        // favours the sign of g (it is halfway one time in six)
+        w.gx6 = fx_mul3(r8, k.gx, k.gx3);
+        w.gy6 = fx_mul3(r8, k.gy, k.gy3);
         if (chi) {
-            hx += fx_mul(r8, fx_split(ax));
-            hy += fx_mul(r8, fx_split(ay));
+            w.gx6 += fx_mul(fx_mul(r8, fx_split(2 * ax)), k.sixth);
+            w.gy6 += fx_mul(fx_mul(r8, fx_split(2 * ay)), k.sixth);
         }
-        Gx = 2 * hx;
-        Gy = 2 * hy;
-        w.gx6 = fx_mul(Gx, k.sixth);
-        w.gy6 = fx_mul(Gy, k.sixth);
-        w.rx = hx - 3 * w.gx6;
-        w.ry = hy - 3 * w.gy6;
     }
     const long long mx = w.jx + (Gx >> 1), my = w.jy + (Gy >> 1);    // rho u = j + G / 2
     const long long mx8 = (long long)((uint64_t)mx << 3), my8 = (long long)((uint64_t)my << 3);
@@ -393,12 +392,6 @@ bool fx_update(const FixedConsts &k, const uint64_t fb[9], bool chi, long long u
         if (!(HERE ? fx_forced_here<false>(k, chi, w) : fx_forced(k, chi, w))) return false;
         de = w.de; dep = w.dep; dqx = w.dqx; dqy = w.dqy; dp = w.dp; dr = w.dr;
         gx6 = w.gx6; gy6 = w.gy6;
-        if (!HERE && k.forced) {
-            f[1] += w.rx;
-            f[3] -= w.rx;
-            f[2] += w.ry;
-            f[4] -= w.ry;
-        }
         ax_o = w.ax;
         ay_o = w.ay;
     } else {
@@ -598,7 +591,7 @@ VPLBM_FX bool fx_equilibrium(const FixedConsts &k, uint64_t rho_b, uint64_t ux_b
         const long long cu = cx * ux + cy * uy, cu2 = (cx ? xx : 0) + (cy ? yy : 0) + 2 * cx * cy * xy;
         const long long poly = ((3 * cu) >> 1) + 18 * cu2 - u15;   // 3 c.u + 9/2 (c.u)^2 - 3/2 u^2, 2^60
         const long long rp = fx_mul(r8, fx_split(2 * poly));        // rho poly, 2^(E - 59)
-        const FxFactor w = a == 0 ? k.w0 : a <= 4 ? k.w1 : k.w2;    // w_a / 2^0, 4/9 < 1/2
+        const FxFactor w = a == 0 ? FX_W0 : a <= 4 ? FX_W1 : FX_W2;
         if (dev) {
             const long long d = drho + rp;
             if ((uint64_t)(d + (1LL << 60)) >= (uint64_t)(1LL << 61)) return false;

@@ -329,11 +329,6 @@ __device__ __forceinline__ float2 acc_shfl_down(float2 a, int off)
 {
     return make_float2(__shfl_down_sync(0xffffffffu, a.x, off), __shfl_down_sync(0xffffffffu, a.y, off));
 }
-__device__ __forceinline__ double acc_shfl(double a, int lane) { return __shfl_sync(0xffffffffu, a, lane); }
-__device__ __forceinline__ float2 acc_shfl(float2 a, int lane)
-{
-    return make_float2(__shfl_sync(0xffffffffu, a.x, lane), __shfl_sync(0xffffffffu, a.y, lane));
-}
 __device__ __forceinline__ double acc_value(double a) { return a; }
 __device__ __forceinline__ double acc_value(float2 a) { return (double)a.x + (double)a.y; }   // exact
 
