@@ -514,9 +514,9 @@ VPLBM_FX bool fx_moments(const FixedConsts &k, const uint64_t fb[9], double &rho
 
 // The same for FP32 / FP16 storage (deviations, as floats).  A deviation has
 // its 24 bits relative to itself, so the sums are on a grid of their own, set
-// by the node's largest one: d 2^(58 - T), 2^T > |d|, on which a float down to
-// 2^-34 of the largest is exact (a node with a smaller one that is not zero,
-// or with a largest one below 2^-92, is left to the FP64 code).  The sums are
+// by the node's largest one: d 2^(56 - T), 2^T > |d|, on which a float down to
+// 2^-31 of the largest is exact (a node with a smaller one that is not zero,
+// or with a largest one below 2^-95, is left to the FP64 code).  The sums are
 // then exact, and u has the precision of a double for any size of the
 // deviations; on the grid of rho0 a deviation of 1e-14 would keep 15 bits.
 VPLBM_FX bool fx_moments_dev(const FixedConsts &k, const float d[9], double &rho_o, double &ux_o, double &uy_o)
@@ -532,20 +532,27 @@ VPLBM_FX bool fx_moments_dev(const FixedConsts &k, const float d[9], double &rho
         low = m - 1u < low ? m - 1u : low;
     }
     const int et = (int)(top >> 23), el = (int)((low + 1u) >> 23);
-    if (k.e < -30 || k.e > 60 || top >= (uint32_t)(124 + k.e) << 23 || (top != 0 && (et < 35 || et - el > 34))) return false;
+    if (k.e < -30 || k.e > 60 || top >= (uint32_t)(124 + k.e) << 23 || (top != 0 && (et < 32 || et - el > 31))) return false;
 #if defined(__CUDA_ARCH__)
 #pragma unroll
 #endif
     for (int a = 0; a < 9; ++a) {
-        const uint32_t b = fx_float_bits(d[a]), s = (uint32_t)et - ((b >> 23) & 0xffu);
-        const long long x = s > 34 || top == 0 ? 0 : (long long)(((uint64_t)((b & 0x7fffffu) | 0x800000u) << 34) >> s);
-        f[a] = (b >> 31) ? -x : x;
+        // a zero has no leading bit; its shift does not matter
+        const uint32_t b = fx_float_bits(d[a]), m = b & 0x7fffffffu, s = (uint32_t)et - (m >> 23);
+        const uint32_t hi = (m & 0x7fffffu) | (m < 0x800000u ? m : 0x800000u);
+#if defined(__CUDA_ARCH__)
+        const uint64_t x = ((uint64_t)(hi >> (s & 31)) << 32) | __funnelshift_r(0u, hi, s);
+#else
+        const uint64_t x = ((uint64_t)hi << 32) >> (s & 31);
+#endif
+        const long long sign = (int)b >> 31;
+        f[a] = ((long long)x ^ sign) - sign;
     }
     const long long sx = f[5] - f[6] - f[7] + f[8], sy = f[5] + f[6] - f[7] - f[8];
-    const long long rs = f[0] + f[1] + f[2] + f[3] + f[4] + f[5] + f[6] + f[7] + f[8];   // below 9 2^58
-    const long long jx = f[1] - f[3] + sx, jy = f[2] - f[4] + sy;                        // below 6 2^58
-    const int T = et - 126, n = k.e - 1 - T;   // to the grid of rho: 2^(E - 59); n >= 2
-    const long long rho = k.rho0 + (n > 62 ? 0 : (rs + (1LL << (n - 1))) >> n);
+    const long long rs = f[0] + f[1] + f[2] + f[3] + f[4] + f[5] + f[6] + f[7] + f[8];   // below 9 2^56
+    const long long jx = f[1] - f[3] + sx, jy = f[2] - f[4] + sy;                        // below 6 2^56
+    const int T = et - 126, n = k.e - 3 - T;   // to the grid of rho: 2^(E - 59)
+    const long long rho = k.rho0 + (n > 62 ? 0 : n > 0 ? (rs + (1LL << (n - 1))) >> n : rs);
     if ((uint64_t)(rho - (1LL << 58)) >= (uint64_t)(1LL << 59)) return false;
     const FxFactor inv = fx_split(fx_recip(rho));   // 2^120 / rho
     auto quotient = [&](long long j) {              // its leading bit to bit 61 first
@@ -553,7 +560,7 @@ VPLBM_FX bool fx_moments_dev(const FixedConsts &k, const float d[9], double &rho
         const uint64_t m = j < 0 ? 0 - (uint64_t)j : (uint64_t)j;
         const int up = fx_clz64(m) - 2;
         const long long q = fx_mul((long long)(m << up), inv);
-        return fx_signed_to(j < 0 ? -q : q, T - k.e - 55 - up);
+        return fx_signed_to(j < 0 ? -q : q, T - k.e - 53 - up);
     };
     rho_o = fx_to(rho, k.e);
     ux_o = quotient(jx);

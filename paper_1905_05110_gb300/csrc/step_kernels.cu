@@ -139,7 +139,7 @@ __global__ void outlet_reset_kernel(const StepParams p)
 //
 // Away from the bodies in fixed point where the node is in range, for the
 // same reason (60 FP64 instructions a node; 2048 x 1024, FP32 storage:
-// us per call to the device 299 -> 41, to page-locked host memory 351 -> 312,
+// us per call to the device 299 -> 40, to page-locked host memory 351 -> 312,
 // of which the link takes 263).
 
 template <int P>
