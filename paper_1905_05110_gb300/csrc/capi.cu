@@ -159,13 +159,15 @@ inline int body_slots(int nb) { return nb > 1 ? nb : 1; }
 // Resident kernel: the tiling, and whether this lattice can take it.
 //
 // The lattice has to fit: one tile on every SM but the tail's, of at most as
-// many nodes as its threads hold (resident_k).  Of the tilings that do, the fewest nodes per
-// thread, then the smallest tile, then the shortest edge.  Tiles are at least
-// 8 nodes wide and high (a lattice narrower than 16 is one tile there), since
-// smaller ones exchange more than they update.  Every lattice that fits takes
-// it unless a kernel was asked for: it was faster than the launches at every
-// size measured, by 4.2x at 97 x 70 (2.1 us a step against 8.9), 3.1x at 512 x
-// 256, 1.8x at 900 x 450 and 1.7x at 1230 x 410, where the registers end it.
+// many nodes as its threads hold (resident_k).  Of the tilings that do, the
+// fewest nodes per thread, then the smallest tile, then the shortest edge.
+// Tiles are at least 8 nodes wide and high (a lattice narrower than 16 is one
+// tile there), since smaller ones exchange more than they update.  Every
+// lattice that fits takes it unless a kernel was asked for or too many streams
+// step such lattices (resident_now): by itself it was faster than the launches
+// at every size measured, by 4.2x at 97 x 70 (2.1 us a step against 8.9), 3.1x
+// at 512 x 256, 1.8x at 900 x 450 and 1.7x at 1230 x 410, where the registers
+// end it.
 bool plan_resident(int nx, int ny, int precision, ResidentPlan *out)
 {
     constexpr int sms = RES_SMS;

@@ -24,7 +24,7 @@
 // Measured (GB300, us per step, best block shape): 2048 x 1024 513 -> 63.5
 // (32.9 k MLUPS, 4.7 TB/s), 256 x 128 28 -> 13.5 (there the launch boundary
 // and the body's sums remain); 2048 x 1024 under a uniform
-// acceleration 114.
+// acceleration 110.
 //
 // Range.  A node takes this path if every population is in
 // [2^(E-32), 2^E), rho in [2^(E-1), 1.5 2^E), |j| < 0.35 2^E and (body

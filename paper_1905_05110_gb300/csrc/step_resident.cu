@@ -50,10 +50,11 @@
 // Measured (GB300, us per step, one-step launches -> this kernel): FP32 256 x
 // 128 with a fixed disk 8.9 -> 2.4, 512 x 256 oscillating disk 8.7 -> 2.8, 512
 // x 256 disk on a spring (free) 14.1 -> 4.7, 700 x 400 9.0 -> 4.3, 1230 x 410
-// 10.5 -> 6.2; FP64 256 x 128 13.6 -> 6.6 (8.1 with the solid-node sums in FP64
+// 10.5 -> 6.2; FP64 256 x 128 13.6 -> 6.5 (8.1 with the solid-node sums in FP64
 // instructions).  What is left: the update itself at
 // 7 nodes a thread (issue slots about half busy), and below 2 nodes a thread
-// the exchange and the three block barriers of a step.
+// the exchange and the three block barriers of a step.  Contexts on streams of
+// their own gain less, since a launch takes every SM (resident_now, capi.cu).
 #define VPLBM_PLAIN_LOADS 1
 #include "vplbm_node.cuh"
 
@@ -1237,6 +1238,8 @@ template <int P, int COLL> cudaError_t launch_pc(const ResidentLaunch &L, cudaSt
         if (L.t.k == 3) return launch_k<P, COLL, 3>(L, stream);
         if (L.t.k == 4) return launch_k<P, COLL, 4>(L, stream);
         if (L.t.k == 5) return launch_k<P, COLL, 5>(L, stream);
+        // six too: a kernel of its own would be 3 to 5 % faster there (1100 x
+        // 400: 5.59 against 5.85 us a step) and is one more to build
         if (L.t.k <= 7) return launch_k<P, COLL, 7>(L, stream);
     }
     return cudaErrorInvalidValue;
